@@ -108,6 +108,7 @@ __global__ void dw_xpay_kernel(float4 *__restrict__ p, const float4 *__restrict_
 // ---- single-block scalar steps -------------------------------------------------
 
 __global__ void finalize_sum_kernel(const double *partials, int n, double *out) {
+  pdl_enter();
   const double s = block_sum_partials(partials, n);
   if (threadIdx.x == 0) *out = s;
 }
@@ -145,8 +146,7 @@ __global__ void cg_start_kernel(const double *partials, int n, SolverScalars *S,
 
 cudaError_t launch_finalize_sum(const double *partials, int n, double *out, cudaStream_t s) {
   note_launch();
-  finalize_sum_kernel<<<1, kReduceThreads, 0, s>>>(partials, n, out);
-  return cudaGetLastError();
+  return launch_pdl(finalize_sum_kernel, 1, kReduceThreads, 0, s, partials, n, out);
 }
 cudaError_t launch_dw_copy(float4 *dst, const float4 *src, int64_t n, cudaStream_t s) {
   note_launch();

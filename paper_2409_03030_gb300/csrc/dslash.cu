@@ -194,8 +194,8 @@ static cudaError_t launch_hop_p(const HopParams &P, bool dag, bool axpy, bool no
 // mul.rn.f32x2 per complex operation halves the instruction issue of a
 // scalar double-word hop, which was bound by issue rather than by the FP32
 // datapath.
-template <bool DAG, bool AXPY, bool NORM, int MINB>
-__global__ void __launch_bounds__(kDwp1Threads, MINB) hop_dwp_kernel(const HopParams P) {
+template <bool DAG, bool AXPY, bool NORM>
+__global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS) hop_dwp_kernel(const HopParams P) {
   extern __shared__ float4 dsm[];
   pdl_enter();
   if (P.guard && *P.guard) return;  // uniform across the grid
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kDwp1Threads, MINB) hop_dwp_kernel(const HopPa
 template <bool DAG, bool AXPY, bool NORM>
 __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS) hop_dwp2_kernel(const HopParams P) {
   extern __shared__ float4 dsm[];
-  pdl_enter();
+  pdl_wait();
   if (P.guard && *P.guard) return;  // uniform across the grid
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t idx = gid >> 1;
@@ -228,15 +228,16 @@ __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS) hop_dwp2_k
   const bool active = idx < P.g.vh;  // the same for both threads of a site
   p2 acc[4][3];
   if (active) {
-    dwp_hop_dirs<DAG, kDwp2Threads>(dsm, reinterpret_cast<const float4 *>(P.in),
-                                     reinterpret_cast<const float4 *>(P.gauge), P.g, P.out_parity, idx, q,
-                                     2, 4, acc);
+    dwp_hop_dirs<DAG, kDwp2Threads, 4, 2>(dsm, reinterpret_cast<const float4 *>(P.in),
+                                                reinterpret_cast<const float4 *>(P.gauge), P.g, P.out_parity,
+                                                (unsigned)idx, q, acc);
   } else {
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[a][c] = p2{0ull, 0ull};
   }
+  pdl_trigger();  // the split grid is less than one wave
   p2 o[6];
   dwp_pair_combine(acc, q, o);  // every lane of the warp takes part
   dwacc nrm{0.f, 0.f};
@@ -268,18 +269,23 @@ bool dw_hop_split(int64_t vh) {
   return vh <= max_vh && vh <= JQCD_DWP_SPLIT_MAX_VH;
 }
 
-// A one-thread grid of at most SMs x JQCD_DWP_SMALL_MIN_BLOCKS blocks takes
-// the form compiled for that occupancy: 184 instead of 166 registers, so
-// fewer dependent chains are serialised to save registers (measured on
-// GB300: 16^4 hop 18.75 -> 13.94 us, its double-word solve 5.34 -> 4.60 ms;
-// at 24^3x48 the same form, at 2 blocks/SM, ran 110.5 against 97.9 us).
+// A one-thread grid of at most SMs x JQCD_DWP_SMALL_BLOCKS blocks is launched
+// with kDwpSmallSmem of shared memory, so that no SM takes a third block.
+// Back to back, each grid's blocks are placed (programmatic launch) while the
+// one before still runs; with room for three, some SMs get three and the grid
+// waits for them.  Measured on GB300 at 16^4: 17.0 us with room for three,
+// 12.8 us for two (13.4 us for the 184-register kernel that two blocks per SM
+// were once cut for); Mhat^dag Mhat p with its norm 63.8 -> 57.2 us, the
+// double-word solve 4.95 -> 4.71 ms.  All hops unrolled took 11.7 us when the
+// same kernel ran back to back, but its code (four kernels of about 90 KB)
+// misses the instruction cache in a real chain: 5.3 ms.
 bool dw_hop_small(int64_t vh) {
   static const int64_t max_vh = [] {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
       return (int64_t)0;
-    return (int64_t)sms * JQCD_DWP_SMALL_MIN_BLOCKS * kDwp1Threads;
+    return (int64_t)sms * JQCD_DWP_SMALL_BLOCKS * kDwp1Threads;
   }();
   return !dw_hop_split(vh) && vh <= max_vh && vh <= JQCD_DWP_SMALL_MAX_VH;
 }
@@ -297,21 +303,18 @@ template <bool DAG, bool AXPY, bool NORM>
 static cudaError_t launch_hop_dw_t(const HopParams &P, cudaStream_t s) {
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
-  auto kern = hop_dwp_kernel<DAG, AXPY, NORM, JQCD_DWP_MIN_BLOCKS>;
-  auto kern_s = hop_dwp_kernel<DAG, AXPY, NORM, JQCD_DWP_SMALL_MIN_BLOCKS>;
+  auto kern = hop_dwp_kernel<DAG, AXPY, NORM>;
   auto kern2 = hop_dwp2_kernel<DAG, AXPY, NORM>;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwp1Smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kern_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwp1Smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwp2Smem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
   if (dw_hop_split(P.g.vh)) return launch_pdl(kern2, dw_hop_blocks(P.g.vh), kDwp2Threads, kDwp2Smem, s, P);
-  if (dw_hop_small(P.g.vh)) return launch_pdl(kern_s, dw_hop_blocks(P.g.vh), kDwp1Threads, kDwp1Smem, s, P);
-  return launch_pdl(kern, dw_hop_blocks(P.g.vh), kDwp1Threads, kDwp1Smem, s, P);
+  return launch_pdl(kern, dw_hop_blocks(P.g.vh), kDwp1Threads, dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s,
+                    P);
 }
 
 static cudaError_t launch_hop_dw(const HopParams &P, bool dag, bool axpy, bool norm, cudaStream_t s) {
@@ -335,6 +338,7 @@ cudaError_t launch_hop(int prec, const HopParams &P, bool dag, bool axpy, bool n
   if (P.fin && (prec == PREC_DW || !norm || !P.fin_S ||
                 hop_norm_partials(prec, P.g.vh) > (unsigned)JQCD_FIN_MAX_BLOCKS))
     return cudaErrorInvalidValue;
+  if (P.g.vh >= kMaxHopSites) return cudaErrorInvalidValue;  // 32-bit neighbour offsets
   switch (prec) {
     case PREC_DW: return launch_hop_dw(P, dag, axpy, norm, s);
     case PREC_F64: return launch_hop_p<PREC_F64>(P, dag, axpy, norm, s);

@@ -69,11 +69,13 @@ __device__ __forceinline__ void two_sum2(f2 a, f2 b, f2 &s, f2 &e) {
   e = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
 }
 
-// a + sg*b lane-wise, sg = +-1 per lane (exact product), unnormalised.
+// a + sg*b lane-wise, sg = +-1 per lane, unnormalised: TwoSum with the sign
+// riding on its fmas (sg*b is exact, so each rounds as the add it replaces);
+// the same result as multiplying b by sg first, one operation fewer.
 __device__ __forceinline__ p2 p2_add_sgn(p2 a, p2 b, f2 sg) {
-  const f2 sb = f2_mul(sg, b.h);
-  f2 s, e;
-  two_sum2(a.h, sb, s, e);
+  const f2 s = f2_fma(sg, b.h, a.h);
+  const f2 nb = f2_sub(a.h, s);  // minus the part of s that is sg*b's
+  const f2 e = f2_add(f2_sub(a.h, f2_add(s, nb)), f2_fma(sg, b.h, nb));
   return p2{s, f2_add(f2_fma(sg, b.l, a.l), e)};
 }
 __device__ __forceinline__ p2 p2_add(p2 a, p2 b) {
@@ -86,6 +88,7 @@ __device__ __forceinline__ p2 p2_norm(p2 a) {  // Fast2Sum per lane
   return p2{s, f2_sub(a.l, f2_sub(s, a.h))};
 }
 __device__ __forceinline__ p2 p2_swap(p2 a) { return p2{f2_swap(a.h), f2_swap(a.l)}; }
+__device__ __forceinline__ p2 p2_neg(p2 a) { return p2{f2_neg(a.h), f2_neg(a.l)}; }
 __device__ __forceinline__ p2 p2_scale_sgn(p2 a, f2 sg) { return p2{f2_mul(sg, a.h), f2_mul(sg, a.l)}; }
 // complex conjugate of a double-word complex number: the sign bits of both
 // words' imaginary lanes flipped (integer ALU, no floating-point operation)

@@ -68,8 +68,8 @@ __device__ __forceinline__ dwacc dwp_store_cg(const p2 (&v)[NC], int k0, const f
   return dwacc{s, __fadd_rn(__fadd_rn(c0, c1), e)};
 }
 
-template <bool XUPD, int MINB>
-__global__ void __launch_bounds__(kDwp1Threads, MINB)
+template <bool XUPD>
+__global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
     hop_dwp_cg_kernel(const HopParams P, const float4 *__restrict__ p, float4 *__restrict__ xs,
                       float4 *__restrict__ r, const float2 *__restrict__ alpha) {
   extern __shared__ float4 dsm[];
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
     hop_dwp2_cg_kernel(const HopParams P, const float4 *__restrict__ p, float4 *__restrict__ xs,
                        float4 *__restrict__ r, const float2 *__restrict__ alpha) {
   extern __shared__ float4 dsm[];
-  pdl_enter();
+  pdl_wait();
   if (P.guard && *P.guard) return;  // uniform across the grid
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t idx = gid >> 1;
@@ -106,15 +106,16 @@ __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
   const bool active = idx < P.g.vh;
   p2 acc[4][3];
   if (active) {
-    dwp_hop_dirs<true, kDwp2Threads>(dsm, reinterpret_cast<const float4 *>(P.in),
-                                      reinterpret_cast<const float4 *>(P.gauge), P.g, P.out_parity, idx, q, 2,
-                                      4, acc);
+    dwp_hop_dirs<true, kDwp2Threads, 4, 2>(dsm, reinterpret_cast<const float4 *>(P.in),
+                                                 reinterpret_cast<const float4 *>(P.gauge), P.g, P.out_parity,
+                                                 (unsigned)idx, q, acc);
   } else {
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[a][c] = p2{0ull, 0ull};
   }
+  pdl_trigger();  // the split grid is less than one wave
   p2 o[6];
   dwp_pair_combine(acc, q, o);
   dwacc nrm{0.f, 0.f};
@@ -194,11 +195,8 @@ static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD, JQCD_DWP_MIN_BLOCKS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwp1Smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD, JQCD_DWP_SMALL_MIN_BLOCKS>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwp1Smem);
+    cudaError_t e = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kDwpSmallSmem);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(hop_dwp2_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kDwp2Smem);
@@ -208,11 +206,8 @@ static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x
   if (dw_hop_split(P.g.vh))
     return launch_pdl(hop_dwp2_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp2Threads, kDwp2Smem, s, P, p, x,
                       r, alpha);
-  if (dw_hop_small(P.g.vh))
-    return launch_pdl(hop_dwp_cg_kernel<XUPD, JQCD_DWP_SMALL_MIN_BLOCKS>, dw_hop_blocks(P.g.vh), kDwp1Threads,
-                      kDwp1Smem, s, P, p, x, r, alpha);
-  return launch_pdl(hop_dwp_cg_kernel<XUPD, JQCD_DWP_MIN_BLOCKS>, dw_hop_blocks(P.g.vh), kDwp1Threads, kDwp1Smem,
-                    s, P, p, x, r, alpha);
+  return launch_pdl(hop_dwp_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp1Threads,
+                    dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P, p, x, r, alpha);
 }
 
 cudaError_t launch_hop_dw_cg(const HopParams &P, const float4 *p, float4 *x, float4 *r,

@@ -77,5 +77,34 @@ __device__ __forceinline__ int64_t hop_neighbour(const Geom &g, int x, int y, in
   return cb_index(g, x, y, z, t);
 }
 
+// Byte offsets (16 x checkerboard index) of the eight neighbours of site idx
+// of parity p, hop d = 2 mu + backward; bit 0 is set on a hop that crosses an
+// antiperiodic time boundary.  32-bit arithmetic throughout: a resident gauge
+// field takes 2688 bytes per site of one parity, so vh < 2^27 on any device
+// (launch_hop refuses more) and 16 idx < 2^31.  Each neighbour is one select
+// of a constant step; the 64-bit coordinates-to-index form took about 25
+// instructions per hop.
+constexpr int64_t kMaxHopSites = (int64_t)1 << 27;
+__device__ __forceinline__ void hop_offsets(const Geom &g, unsigned idx, int p, unsigned (&off)[8]) {
+  const unsigned nxh = g.nxh, ny = g.ny, nz = g.nz;
+  const unsigned xh = idx % nxh;
+  unsigned r = idx / nxh;
+  const unsigned y = r % ny;
+  r /= ny;
+  const unsigned z = r % nz;
+  const unsigned t = r / nz;
+  const bool odd = (y + z + t + p) & 1;  // x = 2 xh + odd
+  const unsigned sz = nxh * ny, st = sz * nz, vh = (unsigned)g.vh;
+  const unsigned neg = g.tanti ? 1u : 0u;
+  const bool tl = t + 1 == (unsigned)g.nt, tf = t == 0;
+  off[0] = 16u * (odd ? (xh + 1 == nxh ? idx + 1 - nxh : idx + 1) : idx);
+  off[1] = 16u * (odd ? idx : (xh == 0 ? idx + nxh - 1 : idx - 1));
+  off[2] = 16u * (y + 1 == ny ? idx + nxh - sz : idx + nxh);
+  off[3] = 16u * (y == 0 ? idx + sz - nxh : idx - nxh);
+  off[4] = 16u * (z + 1 == nz ? idx + sz - st : idx + sz);
+  off[5] = 16u * (z == 0 ? idx + st - sz : idx - sz);
+  off[6] = 16u * (tl ? idx + st - vh : idx + st) | (tl ? neg : 0u);
+  off[7] = 16u * (tf ? idx + vh - st : idx - st) | (tf ? neg : 0u);
+}
 
 }  // namespace jqcd

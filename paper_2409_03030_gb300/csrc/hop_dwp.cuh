@@ -20,9 +20,9 @@ namespace jqcd {
 constexpr int kDwpStageChunks = 12;  // one double-word spinor per thread
 constexpr int kDwpLinkChunks = 9;    // one double-word link per thread and stage
 // one neighbour-spinor stage and two link stages, chunk-major [k][thread],
-// for blocks of nt threads
+// and the eight neighbour offsets (4 bytes each), for blocks of nt threads
 constexpr size_t dwp_smem(int nt = kHopThreads) {
-  return (size_t)(kDwpStageChunks + 2 * kDwpLinkChunks) * nt * 16;
+  return (size_t)(kDwpStageChunks + 2 * kDwpLinkChunks + 2) * nt * 16;
 }
 constexpr size_t kDwpSmem = dwp_smem();
 
@@ -39,11 +39,12 @@ constexpr size_t kDwpSmem = dwp_smem();
 #ifndef JQCD_DWP_MIN_BLOCKS
 #define JQCD_DWP_MIN_BLOCKS 3
 #endif
-// Lattices whose one-thread grid fits in SMs x JQCD_DWP_SMALL_MIN_BLOCKS
-// blocks (16^4) run the same kernel compiled for that many blocks per SM:
-// the register budget, not the occupancy, limits them there.
-#ifndef JQCD_DWP_SMALL_MIN_BLOCKS
-#define JQCD_DWP_SMALL_MIN_BLOCKS 2
+// One-thread grids of at most SMs x JQCD_DWP_SMALL_BLOCKS blocks (16^4) ask
+// for so much shared memory that an SM holds no more than that many: with
+// room for three, the blocks of back-to-back launches crowd some SMs while
+// others run one (dw_hop_small).
+#ifndef JQCD_DWP_SMALL_BLOCKS
+#define JQCD_DWP_SMALL_BLOCKS 2
 #endif
 #ifndef JQCD_DWP2_THREADS
 #define JQCD_DWP2_THREADS 32
@@ -53,34 +54,35 @@ constexpr size_t kDwpSmem = dwp_smem();
 #endif
 constexpr int kDwp1Threads = JQCD_DWP_THREADS;
 constexpr size_t kDwp1Smem = dwp_smem(kDwp1Threads);
+// 227 KB of shared memory per SM, 1 KB of it reserved per block
+constexpr size_t kDwpSmallSmem = (size_t)(227 / JQCD_DWP_SMALL_BLOCKS - 2) * 1024;
+static_assert(kDwpSmallSmem >= kDwp1Smem, "the limit only pads the stages");
 constexpr int kDwp2Threads = JQCD_DWP2_THREADS;
 constexpr size_t kDwp2Smem = dwp_smem(kDwp2Threads);
 
-// Issue the copies of the neighbour spinor of one hop into its stage (NT:
-// threads per block, the stride of the chunk-major stage).
-template <int NT = kHopThreads>
-__device__ __forceinline__ void stage_hop_p(float4 *st, const float4 *in, int64_t vh, int64_t nb) {
-  const int tid = threadIdx.x;
+// Issue the copies of a spinor (byte offset off) into its stage column st
+// (NT: threads per block, the stride of the chunk-major stage).  The chunk
+// planes in + k vh are uniform over the grid, so the per-thread part of every
+// address is the one 32-bit offset.  L1: through L1, where the neighbours of a
+// few resident warps find each other's spinors, or past it.
+template <int NT, bool L1>
+__device__ __forceinline__ void stage_hop_p(float4 *st, const float4 *in, int64_t vh, unsigned off) {
 #pragma unroll
-  for (int k = 0; k < 12; ++k) cp_async16(st + k * NT + tid, in + k * vh + nb, true);
+  for (int k = 0; k < 12; ++k) cp_async16(st + k * NT, reinterpret_cast<const char *>(in + k * vh) + off, L1);
 }
 
 // Issue the copies of the link of hop d (mu = d/2, backward when d is odd)
-// into a link stage, element (a, b) at chunk 3a + b: U_mu(x) for a forward
-// hop, the transpose of U_mu(x - mu) (conjugated at use) for a backward one.
+// into a link stage column, element (a, b) at chunk 3a + b: U_mu(x) for a
+// forward hop (own: byte offset of x), U_mu(x - mu) for a backward one (nb:
+// byte offset of the neighbour); transposed and conjugated at use.
 template <int NT = kHopThreads>
 __device__ __forceinline__ void stage_link_p(float4 *st, const float4 *gauge, int64_t vh, int p, int d,
-                                             int64_t idx, int64_t nb) {
-  const int tid = threadIdx.x;
-  const int mu = d >> 1;
+                                             unsigned own, unsigned nb) {
   const bool bwd = (d & 1) != 0;
-  const float4 *L = gauge + (size_t)(((bwd ? 1 - p : p) * 4 + mu) * 9) * vh + (bwd ? nb : idx);
-  const int sa = bwd ? 1 : 3, sb = bwd ? 3 : 1;
+  const float4 *L = gauge + (int64_t)(((bwd ? 1 - p : p) * 4 + (d >> 1)) * 9) * vh;
+  const unsigned off = bwd ? nb : own;
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b)
-      cp_async16(st + (a * 3 + b) * NT + tid, L + (int64_t)(a * sa + b * sb) * vh, false);
+  for (int k = 0; k < 9; ++k) cp_async16(st + k * NT, reinterpret_cast<const char *>(L + k * vh) + off, false);
 }
 
 __device__ __forceinline__ p2 ld_p2(const float4 *p) {
@@ -232,57 +234,83 @@ __device__ __forceinline__ void reconstruct_half_mu(int mu, const p2 (&r)[3], p2
   }
 }
 
-// acc = the sum over the hops d = d0, d0 + dstep, ... (nd of them; hop d
-// has mu = d/2 and is backward when d is odd) of H_{p,1-p} in at output site
-// idx of parity p (DAG: the adjoint hop), unnormalised double-word
-// accumulators.  All eight hops (d0 = 0, dstep = 1, nd = 8) give
-// (H_{p,1-p} in)(idx).  dsm: this block's kDwpSmem bytes of shared memory;
-// blockDim.x must be NT.
+// acc = the sum over the ND hops d = d0, d0 + DSTEP, ... (hop d has mu = d/2
+// and is backward when d is odd) of H_{p,1-p} in at output site idx of parity
+// p (DAG: the adjoint hop), unnormalised double-word accumulators.  All eight
+// hops (d0 = 0, DSTEP = 1, ND = 8) give (H_{p,1-p} in)(idx).  dsm: this
+// block's dwp_smem(NT) bytes of shared memory; blockDim.x must be NT.
 //
-// Copies run one hop ahead: the links of the next hop are issued when hop d
+// Copies run one hop ahead: the link of the next hop is issued when hop d
 // starts (two link stages), the neighbour spinor of the next hop as soon as
 // hop d's has been read into registers and projected (one stage).  Every
 // thread reads and overwrites only its own column, so no block barrier is
 // needed; the completed-group wait of each hop covers both of its copies.
-template <bool DAG, int NT = kHopThreads>
+//
+// All eight hops in one thread (DSTEP 1): a runtime loop, whose body exists
+// once in the instruction stream; the neighbour offsets wait in shared
+// memory, one load per hop.  Computing each hop's neighbour and its 64-bit
+// chunk addresses in the loop instead took 49 of 748 instructions per hop and
+// warp, and the kernel is bound by issue and dependency latency at 12 warps
+// per SM.  With the spinor copies past L1 (cp.async.cg: three blocks' stages
+// leave L1 about 56 KB, less than the spinor bytes in flight, so allocating
+// there limited them): 97.9 -> 91.5 us at 24^3x48, 286.8 -> 265.1 us at
+// 32^3x64 (5.57 and 6.08 TB/s algorithmic, 82% and 90% of the measured copy
+// bandwidth).
+// Every other hop (DSTEP 2, two threads per site on small lattices): the four
+// hops unrolled with their offsets in registers; each SM's few warps are bound
+// by the latency of their own chain, and their directions are then constants
+// (12^4 solve 3.08 -> 2.99 ms); L1 is large beside their small stages and keeps
+// the spinors (past L1 the 14^4 solve takes 4.48 instead of 3.75 ms).
+template <bool DAG, int NT, int ND, int DSTEP>
 __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, const float4 *gauge,
-                                             const Geom &g, int p, int64_t idx, int d0, int dstep,
-                                             int nd, p2 (&acc)[4][3]) {
+                                             const Geom &g, int p, unsigned idx, int d0,
+                                             p2 (&acc)[4][3]) {
   const int64_t vh = g.vh;
-  int x, y, z, t;
-  cb_coords(g, idx, p, x, y, z, t);
+  const int tid = threadIdx.x;
+  float4 *const spn = dsm + tid;                     // this thread's column of the spinor stage
+  float4 *const lnk = spn + kDwpStageChunks * NT;    // and of the two link stages
+  unsigned *const tab = reinterpret_cast<unsigned *>(dsm + (kDwpStageChunks + 2 * kDwpLinkChunks) * NT) + tid;
+  unsigned off[8];
+  hop_offsets(g, idx, p, off);
+  if (DSTEP == 1) {
+#pragma unroll
+    for (int d = 0; d < 8; ++d) tab[d * NT] = off[d];
+  }
+  auto offset = [&](int j) -> unsigned {  // of the j-th hop
+    if (DSTEP == 1) return tab[j * NT];
+    return d0 ? off[(2 * j + 1) & 7] : off[(2 * j) & 7];
+  };
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[a][c] = p2{0ull, 0ull};
-  const int tid = threadIdx.x;
-  float4 *const lnk = dsm + kDwpStageChunks * NT;  // two link stages
-  bool neg_next;
-  int64_t nb = hop_neighbour(g, x, y, z, t, d0, neg_next);
-  stage_hop_p<NT>(dsm, in, vh, nb);
-  stage_link_p<NT>(lnk, gauge, vh, p, d0, idx, nb);
+  const unsigned own = idx * 16u;
+  unsigned next = offset(0);
+  stage_hop_p<NT, DSTEP == 2>(spn, in, vh, next & ~1u);
+  stage_link_p<NT>(lnk, gauge, vh, p, d0, own, next & ~1u);
   cp_async_commit();
-#pragma unroll 1
-  for (int j = 0; j < nd; ++j) {
-    const int d = d0 + j * dstep;
-    const bool neg = neg_next;
-    const int mu = d >> 1;
+#pragma unroll(DSTEP == 2 ? ND : 1)
+  for (int j = 0; j < ND; ++j) {
+    const int d = DSTEP == 1 ? j : d0 + j * DSTEP;
+    const bool neg = next & 1u;
+    const int mu = DSTEP == 2 ? j : d >> 1;
     const bool bwd = (d & 1) != 0;
-    const bool more = j + 1 < nd;
+    const bool more = j + 1 < ND;
     if (more) {  // the other link stage was read during the previous hop
-      nb = hop_neighbour(g, x, y, z, t, d + dstep, neg_next);
-      stage_link_p<NT>(lnk + ((j + 1) & 1) * kDwpLinkChunks * NT, gauge, vh, p, d + dstep, idx, nb);
+      next = offset(j + 1);
+      stage_link_p<NT>(lnk + ((j + 1) & 1) * kDwpLinkChunks * NT, gauge, vh, p, d + DSTEP, own, next & ~1u);
     }
     cp_async_commit();
     cp_async_wait1();  // this thread's spinor and link copies of hop d have landed
     p2 psi[4][3];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) psi[k / 3][k % 3] = ld_p2(dsm + k * NT + tid);
+    for (int k = 0; k < 12; ++k) psi[k / 3][k % 3] = ld_p2(spn + k * NT);
     p2 W[3][3];
-    {
-      const float4 *ls = lnk + (j & 1) * kDwpLinkChunks * NT + tid;
+    {  // U_mu(x), or the transpose of U_mu(x - mu)
+      const float4 *ls = lnk + (j & 1) * kDwpLinkChunks * NT;
+      const int sa = bwd ? NT : 3 * NT, sb = bwd ? 3 * NT : NT;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) W[k / 3][k % 3] = ld_p2(ls + k * NT);
+      for (int k = 0; k < 9; ++k) W[k / 3][k % 3] = ld_p2(ls + (k / 3) * sa + (k % 3) * sb);
     }
     const float S = (bwd != DAG) ? 1.f : -1.f;
     p2 h[2][3];
@@ -292,14 +320,13 @@ __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, cons
       case 2: project_p<2>(psi, h, S); break;
       default: project_p<3>(psi, h, S);
     }
-    if (more) stage_hop_p<NT>(dsm, in, vh, nb);  // the spinor stage has been read
+    if (more) stage_hop_p<NT, DSTEP == 2>(spn, in, vh, next & ~1u);  // the spinor stage has been read
     cp_async_commit();
     if (neg) {
-      const f2 mm = f2_make(-1.f, -1.f);
 #pragma unroll
       for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) h[a][c] = p2_scale_sgn(h[a][c], mm);
+        for (int c = 0; c < 3; ++c) h[a][c] = p2_neg(h[a][c]);
     }
     if (bwd) {
       // conjugation of the adjoint link on backward hops only, by sign bits
@@ -323,7 +350,7 @@ __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, cons
 template <bool DAG, int NT = kHopThreads>
 __device__ __forceinline__ void dwp_hop_site(float4 *dsm, const float4 *in, const float4 *gauge,
                                              const Geom &g, int p, int64_t idx, p2 (&acc)[4][3]) {
-  dwp_hop_dirs<DAG, NT>(dsm, in, gauge, g, p, idx, 0, 1, 8, acc);
+  dwp_hop_dirs<DAG, NT, 8, 1>(dsm, in, gauge, g, p, (unsigned)idx, 0, acc);
 }
 
 // Two threads per output site (lanes 2i and 2i + 1 of a warp, q = lane & 1):

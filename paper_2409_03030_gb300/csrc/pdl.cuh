@@ -12,10 +12,18 @@
 
 namespace jqcd {
 
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  pdl_wait();
+  pdl_trigger();
 }
+// A grid of less than one wave triggers after its main work instead (pdl_wait
+// first, pdl_trigger near the end): triggered at once, the next grid's blocks
+// take the free slots of SMs that still run this one, so some SMs end up with
+// more of its blocks than others and the whole grid waits for those (measured
+// on GB300: 14^4 double-word hop 14.25 us with the trigger first, 10.63 us
+// with it last).
 
 // kern<<<grid, block, smem, s>>>(args...) with programmatic stream
 // serialization allowed; kern must call pdl_enter() first.
