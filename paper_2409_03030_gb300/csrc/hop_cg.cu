@@ -25,12 +25,12 @@ namespace jqcd {
 namespace {
 
 // q = a*w + b*v is (Ap)(idx) for the NC components k0 .. k0 + NC - 1 of the
-// site; x += alpha p (XUPD) and r -= alpha q in place; returns their
+// site; x += alpha p in place (XUPD) and r = r_in - alpha q; returns its
 // contribution to ||r||^2.  Every operand is a 16-byte double-word chunk.
 template <bool XUPD, int NC>
 __device__ __forceinline__ dwacc dwp_store_cg(const p2 (&v)[NC], int k0, const float4 *__restrict__ w_base,
                                               const float4 *__restrict__ p_base,
-                                              float4 *__restrict__ x_base, float4 *__restrict__ r_base,
+                                              float4 *__restrict__ x_base, const float4 *r_in, float4 *r_base,
                                               int64_t vh, int64_t idx, float2 a_split, float2 b_split,
                                               float2 alpha) {
   idx += (int64_t)k0 * vh;
@@ -41,11 +41,12 @@ __device__ __forceinline__ dwacc dwp_store_cg(const p2 (&v)[NC], int k0, const f
   const ulonglong2 *__restrict__ wp = reinterpret_cast<const ulonglong2 *>(w_base) + idx;
   const ulonglong2 *__restrict__ pp = reinterpret_cast<const ulonglong2 *>(p_base) + idx;
   ulonglong2 *__restrict__ xp = reinterpret_cast<ulonglong2 *>(x_base) + idx;
-  ulonglong2 *__restrict__ rp = reinterpret_cast<ulonglong2 *>(r_base) + idx;
+  const ulonglong2 *ri = reinterpret_cast<const ulonglong2 *>(r_in) + idx;  // may be rp
+  ulonglong2 *rp = reinterpret_cast<ulonglong2 *>(r_base) + idx;
   acc2 nq{0ull, 0ull};
 #pragma unroll
   for (int k = 0; k < NC; ++k) {
-    const ulonglong2 wv = __ldg(wp + k * vh), rv = rp[k * vh];
+    const ulonglong2 wv = __ldg(wp + k * vh), rv = ri[k * vh];
     acc2 R = acc2_first(Bm, p2_norm(v[k]));
     acc2_mad(R, Am, p2{wv.x, wv.y});
     const p2 q = p2_norm(acc2_get(R));
@@ -71,7 +72,7 @@ __device__ __forceinline__ dwacc dwp_store_cg(const p2 (&v)[NC], int k0, const f
 template <bool XUPD>
 __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
     hop_dwp_cg_kernel(const HopParams P, const float4 *__restrict__ p, float4 *__restrict__ xs,
-                      float4 *__restrict__ r, const float2 *__restrict__ alpha) {
+                      const float4 *r_in, float4 *r, const float2 *__restrict__ alpha) {
   extern __shared__ float4 dsm[];
   pdl_enter();
   if (P.guard && *P.guard) return;  // uniform across the grid
@@ -84,7 +85,7 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
     p2 v[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) v[k] = acc[k / 3][k % 3];
-    nrm = dwp_store_cg<XUPD, 12>(v, 0, reinterpret_cast<const float4 *>(P.x), p, xs, r, P.g.vh, idx,
+    nrm = dwp_store_cg<XUPD, 12>(v, 0, reinterpret_cast<const float4 *>(P.x), p, xs, r_in, r, P.g.vh, idx,
                                  P.a_split, P.b_split, *alpha);
   }
   const double s = block_sum_dw(nrm);
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
 template <bool XUPD>
 __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
     hop_dwp2_cg_kernel(const HopParams P, const float4 *__restrict__ p, float4 *__restrict__ xs,
-                       float4 *__restrict__ r, const float2 *__restrict__ alpha) {
+                       const float4 *r_in, float4 *r, const float2 *__restrict__ alpha) {
   extern __shared__ float4 dsm[];
   pdl_wait();
   if (P.guard && *P.guard) return;  // uniform across the grid
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
   dwp_pair_combine(acc, q, o);
   dwacc nrm{0.f, 0.f};
   if (active)
-    nrm = dwp_store_cg<XUPD, 6>(o, 6 * q, reinterpret_cast<const float4 *>(P.x), p, xs, r, P.g.vh, idx,
+    nrm = dwp_store_cg<XUPD, 6>(o, 6 * q, reinterpret_cast<const float4 *>(P.x), p, xs, r_in, r, P.g.vh, idx,
                                 P.a_split, P.b_split, *alpha);
   const double s = block_sum_dw(nrm);
   if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
@@ -190,8 +191,8 @@ cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, const void *p, float4
 }
 
 template <bool XUPD>
-static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x, float4 *r, const float2 *alpha,
-                                  cudaStream_t s) {
+static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x, const float4 *r_in, float4 *r,
+                                  const float2 *alpha, cudaStream_t s) {
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
   if (!configured) {
@@ -205,18 +206,19 @@ static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x
   }
   if (dw_hop_split(P.g.vh))
     return launch_pdl(hop_dwp2_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp2Threads, kDwp2Smem, s, P, p, x,
-                      r, alpha);
+                      r_in, r, alpha);
   return launch_pdl(hop_dwp_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp1Threads,
-                    dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P, p, x, r, alpha);
+                    dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P, p, x, r_in, r, alpha);
 }
 
 cudaError_t launch_hop_dw_cg(const HopParams &P, const float4 *p, float4 *x, float4 *r,
                              const SolverScalars *S, cudaStream_t s) {
-  return launch_dw_cg_t<true>(P, p, x, r, &S->alpha_dw, s);
+  return launch_dw_cg_t<true>(P, p, x, r, r, &S->alpha_dw, s);
 }
 
-cudaError_t launch_hop_dw_r(const HopParams &P, float4 *r, const float2 *alpha_dw, cudaStream_t s) {
-  return launch_dw_cg_t<false>(P, nullptr, nullptr, r, alpha_dw, s);
+cudaError_t launch_hop_dw_r(const HopParams &P, const float4 *r_in, float4 *r, const float2 *alpha_dw,
+                            cudaStream_t s) {
+  return launch_dw_cg_t<false>(P, nullptr, nullptr, r_in, r, alpha_dw, s);
 }
 
 }  // namespace jqcd

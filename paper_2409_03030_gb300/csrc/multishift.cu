@@ -14,6 +14,12 @@
 //   beta_i^k  = beta^k (zeta_i^{k+1} / zeta_i^k)^2, p_i = zeta_i^{k+1} r + beta_i^k p_i
 // Shift i stops (x_i frozen) once |zeta_i| |r| <= tol |rhs|; the loop ends
 // when every shift has.  Scalars live on the device; the host polls.
+//
+// The shifted recurrences never feed back into the base one, so their vectors
+// are not touched in every iteration: up to kMsBlock residuals r_j are kept,
+// the coefficients of each step are recorded, and one pass then applies all
+// the recorded steps to x_i and p_i in registers (the same operations in the
+// same order, so the same bits).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -23,6 +29,7 @@
 #include <vector>
 
 #include "dw.cuh"
+#include "dw2.cuh"
 #include "kernels.h"
 #include "multishift.h"
 #include "pdl.cuh"
@@ -71,10 +78,9 @@ __global__ void ms_start_kernel(const double *partials, int n, MsScalars *S, dou
     S->max_iters = max_iters;
     S->done = 0;
     S->halt = 0;
-    S->final_x = 0;
     for (int i = 0; i < S->nshift; ++i) {
       S->zeta_prev[i] = S->zeta[i] = S->zeta_next[i] = 1.0;
-      S->alpha_s[i] = S->beta_s[i] = 0.0;
+      S->alpha_s[i] = 0.0;
       S->active[i] = rhs2 > 0.0;
       S->conv_iter[i] = 0;
     }
@@ -85,98 +91,167 @@ __global__ void ms_start_kernel(const double *partials, int n, MsScalars *S, dou
   }
 }
 
-__global__ void ms_alpha_kernel(const double *partials, int n, MsScalars *S) {
+// Thread i takes the recurrences of shift i (a loop over the shifts in one
+// thread put its chain of FP64 divisions on the iteration's critical path:
+// 11.9 us per step for 8 shifts).
+__global__ void ms_alpha_kernel(const double *partials, int n, MsScalars *S, MsSteps *B, int slot) {
+  __shared__ double sh_pap;
   pdl_enter();
-  if (S->halt) {  // a queued iteration after the halt: the last x_i update is done
-    if (threadIdx.x == 0) S->final_x = 0;
+  if (slot == 0 && threadIdx.x == 0) B->n = 0;  // the last record has been applied
+  if (S->halt) return;
+  const double v = sum_partials(partials, n);
+  if (threadIdx.x == 0) sh_pap = v;
+  __syncthreads();
+  const double pAp = sh_pap;
+  if (!(pAp > 0.0) || !isfinite(pAp)) {
+    if (threadIdx.x == 0) { S->done = 2; S->halt = 1; }
     return;
   }
-  const double pAp = sum_partials(partials, n);
-  if (threadIdx.x == 0) {
-    if (!(pAp > 0.0) || !isfinite(pAp)) { S->done = 2; S->halt = 1; return; }
-    const double a = S->rr / pAp, ap = S->alpha_prev, b = S->beta;
+  const double a = S->rr / pAp, ap = S->alpha_prev, b = S->beta;
+  const int i = threadIdx.x;
+  if (i < S->nshift && S->active[i]) {
+    const double z = S->zeta[i], zp = S->zeta_prev[i];
+    const double zn = z * zp * ap / (a * b * (zp - z) + zp * ap * (1.0 + S->sigma[i] * a));
+    S->zeta_next[i] = zn;
+    S->alpha_s[i] = a * zn / z;
+  }
+  if (i == 0) {
     S->alpha = a;
     const float ah = __double2float_rn(a);
     S->alpha_dw = make_float2(ah, __double2float_rn(a - (double)ah));
-    for (int i = 0; i < S->nshift; ++i) {
-      if (!S->active[i]) continue;
-      const double z = S->zeta[i], zp = S->zeta_prev[i];
-      const double zn = z * zp * ap / (a * b * (zp - z) + zp * ap * (1.0 + S->sigma[i] * a));
-      S->zeta_next[i] = zn;
-      S->alpha_s[i] = a * zn / z;
-    }
   }
 }
 
-__global__ void ms_beta_kernel(const double *partials, int n, MsScalars *S) {
+__device__ __forceinline__ float2 split_pair(double v) {
+  const float h = __double2float_rn(v);
+  return make_float2(h, __double2float_rn(v - (double)h));
+}
+
+__global__ void ms_beta_kernel(const double *partials, int n, MsScalars *S, MsSteps *B, int slot) {
+  __shared__ double sh_rr;
   pdl_enter();
   if (S->halt) return;
-  const double rr_new = sum_partials(partials, n);
-  if (threadIdx.x == 0) {
-    S->iters += 1;
-    if (!isfinite(rr_new)) { S->done = 2; S->halt = 1; return; }
-    const double b = rr_new / S->rr;
-    int any = 0;
-    for (int i = 0; i < S->nshift; ++i) {
-      S->xact[i] = S->active[i];
-      if (!S->active[i]) continue;
+  const double v = sum_partials(partials, n);
+  if (threadIdx.x == 0) sh_rr = v;
+  __syncthreads();
+  const double rr_new = sh_rr;
+  const int iter = S->iters + 1;
+  const bool last = iter >= S->max_iters;
+  const bool finite = isfinite(rr_new);
+  const double b = rr_new / S->rr;
+  const int i = threadIdx.x;
+  int running = 0;  // this thread's shift goes on
+  if (finite && i < S->nshift) {
+    const bool act = S->active[i] != 0;
+    float2 al = make_float2(0.f, 0.f), ze = al, be = al;
+    if (act) {
       const double z = S->zeta[i], zn = S->zeta_next[i];
-      S->beta_s[i] = b * (zn / z) * (zn / z);
+      al = split_pair(S->alpha_s[i]);
+      ze = split_pair(zn);
+      be = split_pair(b * (zn / z) * (zn / z));
       S->zeta_prev[i] = z;
       S->zeta[i] = zn;
       if (zn * zn * rr_new <= S->stop_rr) {
         S->active[i] = 0;
-        S->conv_iter[i] = S->iters;
+        S->conv_iter[i] = iter;
       } else {
-        any = 1;
+        running = 1;
       }
     }
+    B->alpha[slot][i] = al;
+    B->zeta[slot][i] = ze;
+    B->beta[slot][i] = be;
+    B->xact[slot][i] = act;
+    B->pact[slot][i] = running && !last;
+  }
+  const int any = __syncthreads_or(running);  // every read of S->rr, S->iters is above
+  if (threadIdx.x == 0) {
+    S->iters = iter;
+    if (!finite) { S->done = 2; S->halt = 1; return; }
+    B->n = slot + 1;
     S->beta = b;
     S->alpha_prev = S->alpha;
     S->rr = rr_new;
-    if (!any) { S->done = 1; S->halt = 1; S->final_x = 1; }
-    else if (S->iters >= S->max_iters) { S->done = 3; S->halt = 1; S->final_x = 1; }
+    if (!any) { S->done = 1; S->halt = 1; }
+    else if (last) { S->done = 3; S->halt = 1; }
   }
 }
 
-// After beta: x_i += alpha_i p_i for the shifts active in this iteration
-// (xact; alpha_i from this iteration's alpha step) and p_i = zeta_i r +
-// beta_i p_i for those still active, p = r + beta p: each p_i is read once.
-// Runs while the solve iterates, and once more after the beta step that
-// halted it (final_x).
-__global__ void ms_xp_kernel(float4 *__restrict__ pb, const float4 *__restrict__ r, MsVectors V, int64_t n,
-                             const MsScalars *S) {
-  __shared__ float4 cp[kMsMaxShifts];  // (zeta.h, zeta.l, beta.h, beta.l)
-  __shared__ float2 cx[kMsMaxShifts];  // alpha_i (h, l)
-  __shared__ int ax[kMsMaxShifts], ap[kMsMaxShifts];
+// p = r + beta p of the base system
+__global__ void ms_p_kernel(float4 *__restrict__ pb, const float4 *__restrict__ r, int64_t n, const MsScalars *S) {
   pdl_enter();
-  if (S->halt && !S->final_x) return;  // uniform across the grid
-  const int ns = S->nshift;
-  for (int i = threadIdx.x; i < ns; i += blockDim.x) {
-    const double z = S->zeta[i], b = S->beta_s[i], a = S->alpha_s[i];
-    const float zh = __double2float_rn(z), bh = __double2float_rn(b), ah = __double2float_rn(a);
-    cp[i] = make_float4(zh, __double2float_rn(z - (double)zh), bh, __double2float_rn(b - (double)bh));
-    cx[i] = make_float2(ah, __double2float_rn(a - (double)ah));
-    ax[i] = S->xact[i];
-    ap[i] = S->active[i] && !S->halt;
-  }
-  __syncthreads();
+  if (S->halt) return;  // uniform across the grid
   const dw beta = dw_from_double(S->beta);
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
     dw rr, ri, pr, pi;
     dwc_unpack(r[q], rr, ri);
     dwc_unpack(pb[q], pr, pi);
     pb[q] = dwc_pack(dw_add(rr, dw_mul(beta, pr)), dw_add(ri, dw_mul(beta, pi)));
+  }
+}
+
+__device__ __forceinline__ p2 ld_chunk(const float4 *p) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+  return p2{v.x, v.y};
+}
+__device__ __forceinline__ mul2 bcast(float2 c) { return mul2{f2_make(c.x, c.x), f2_make(c.y, c.y)}; }
+// c v for a real double-word scalar c, normalised (dw_mul on both lanes)
+__device__ __forceinline__ p2 p2_scale(const mul2 &c, p2 v) { return p2_norm(acc2_get(acc2_first(c, v))); }
+
+// The recorded steps of every shift: per element, the residuals of the block
+// are loaded once, then x_i and p_i of each shift are read, taken through all
+// the steps in registers and written back.  An update in every iteration
+// moved 4 streams per running shift each time and was bound by HBM (285.6 us
+// an iteration for 8 shifts at 24^3x48); a block of eight moves them once (610
+// us, 76 us an iteration) and the solve went from 56.2 to 40.7 ms.
+__global__ void __launch_bounds__(kBlasThreads)
+    ms_steps_kernel(MsVectors V, MsResiduals R, int64_t n, const MsScalars *__restrict__ S,
+                    const MsSteps *__restrict__ B) {
+  __shared__ float4 cp[kMsMaxShifts][kMsBlock];  // (zeta, beta) of a step
+  __shared__ float2 cx[kMsMaxShifts][kMsBlock];  // alpha
+  __shared__ int nx[kMsMaxShifts], np[kMsMaxShifts];  // steps of x_i and of p_i (each shift's come first)
+  pdl_enter();
+  const int m = B->n;
+  if (m == 0) return;  // uniform across the grid
+  const int ns = S->nshift;
+  for (int t = threadIdx.x; t < ns * m; t += blockDim.x) {
+    const int i = t / m, j = t % m;
+    const float2 z = B->zeta[j][i], b = B->beta[j][i];
+    cp[i][j] = make_float4(z.x, z.y, b.x, b.y);
+    cx[i][j] = B->alpha[j][i];
+  }
+  for (int i = threadIdx.x; i < ns; i += blockDim.x) {
+    int a = 0, c = 0;
+    for (int j = 0; j < m; ++j) {
+      a += B->xact[j][i];
+      c += B->pact[j][i];
+    }
+    nx[i] = a;
+    np[i] = c;
+  }
+  __syncthreads();
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+    p2 r[kMsBlock];
+#pragma unroll
+    for (int j = 0; j < kMsBlock; ++j) r[j] = j < m ? ld_chunk(R.r[j] + q) : p2{0ull, 0ull};
+#pragma unroll 1
     for (int i = 0; i < ns; ++i) {
-      if (!ax[i]) continue;
-      dwc_unpack(V.p[i][q], pr, pi);
-      const dw a = dw_make(cx[i].x, cx[i].y);
-      dw xr, xi;
-      dwc_unpack(V.x[i][q], xr, xi);
-      V.x[i][q] = dwc_pack(dw_add(xr, dw_mul(a, pr)), dw_add(xi, dw_mul(a, pi)));
-      if (!ap[i]) continue;
-      const dw z = dw_make(cp[i].x, cp[i].y), b = dw_make(cp[i].z, cp[i].w);
-      V.p[i][q] = dwc_pack(dw_add(dw_mul(z, rr), dw_mul(b, pr)), dw_add(dw_mul(z, ri), dw_mul(b, pi)));
+      const int a = nx[i], c = np[i];
+      if (a == 0) continue;
+      float4 *xp = V.x[i] + q, *pp = V.p[i] + q;
+      p2 x = ld_chunk(xp), p = ld_chunk(pp);
+#pragma unroll
+      for (int j = 0; j < kMsBlock; ++j) {
+        if (j >= a) break;  // uniform over the block
+        x = p2_norm(p2_add(x, p2_scale(bcast(cx[i][j]), p)));
+        if (j < c) {
+          const float4 w = cp[i][j];
+          p = p2_norm(p2_add(p2_scale(bcast(make_float2(w.x, w.y)), r[j]),
+                             p2_scale(bcast(make_float2(w.z, w.w)), p)));
+        }
+      }
+      *reinterpret_cast<ulonglong2 *>(xp) = make_ulonglong2(x.h, x.l);
+      if (c > 0) *reinterpret_cast<ulonglong2 *>(pp) = make_ulonglong2(p.h, p.l);
     }
   }
 }
@@ -211,8 +286,30 @@ cudaError_t GaugeEntry::ensure_multishift(int nshift) {
     if (e == cudaSuccess) ms_p.push_back(p);
   }
   if (e == cudaSuccess && !ms_S) e = alloc_t(&ms_S, sizeof(MsScalars));
+  if (e == cudaSuccess && !ms_B) e = alloc_t(&ms_B, sizeof(MsSteps));
   if (e == cudaSuccess && !ms_S_host) e = cudaMallocHost(&ms_S_host, sizeof(MsScalars));
   return e;
+}
+
+// Residuals of a block of iterations beside vr: as many as up to kMsBlock - 1
+// that each take no more than a sixteenth of the free memory (blocks are
+// shorter with fewer; GaugeEntry::alloc gives them back when it runs out).
+void GaugeEntry::ensure_ms_ring() {
+  const size_t half = spinor_parity_bytes(PREC_DW, g.vh);
+  while ((int)ms_r.size() < kMsBlock - 1) {
+    size_t free_b = 0, total = 0;
+    void *p = nullptr;
+    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess || half > free_b / 16 || cudaMalloc(&p, half) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    ms_r.push_back((float4 *)p);
+  }
+}
+
+void GaugeEntry::drop_ms_ring() {
+  for (float4 *p : ms_r) cudaFree(p);
+  ms_r.clear();
 }
 
 jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshift, const double *shifts,
@@ -240,11 +337,20 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
     return JQCD_EINVAL;
   }
   CKM(G.ensure_multishift(nshift));
+  G.ensure_ms_ring();
   const int64_t vh = G.g.vh;
   const int64_t n = 12 * vh;  // complex double-word numbers of one parity
   const int nblas = (int)blas_blocks(n);
   const int nhop = (int)dw_hop_blocks(vh);  // partials of the double-word hops
-  float4 *rhs = G.vec_even(G.vrhs), *r = G.vec_even(G.vr), *pb = G.vec_even(G.vp), *Ap = G.vec_even(G.vAp);
+  float4 *rhs = G.vec_even(G.vrhs), *pb = G.vec_even(G.vp), *Ap = G.vec_even(G.vAp);
+  // step j of a block writes its residual to ring[j]
+  const int nring = 1 + (int)G.ms_r.size();
+  float4 *ring[kMsBlock];
+  MsResiduals R;
+  memset(&R, 0, sizeof R);
+  for (int j = 0; j < nring; ++j) R.r[j] = ring[j] = j + 1 < nring ? G.ms_r[j] : G.vec_even(G.vr);
+  const float4 *r_last = ring[nring - 1];  // the newest residual
+  MsSteps *B = G.ms_B;
   MsVectors V;
   memset(&V, 0, sizeof V);
   for (int i = 0; i < nshift; ++i) {
@@ -260,7 +366,8 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
   CKM(cudaMemcpyAsync(S, H, sizeof(MsScalars), cudaMemcpyHostToDevice, s));
   CKM(launch_dw_norm2(rhs, n, G.partials, s));
   CKM(launch_ms_start(G.partials, nblas, S, P.tol * P.tol, P.maxiter, s));
-  CKM(launch_dw_copy(r, rhs, n, s));
+  CKM(cudaMemsetAsync(&B->n, 0, sizeof B->n, s));
+  CKM(launch_dw_copy(ring[nring - 1], rhs, n, s));
   CKM(launch_dw_copy(pb, rhs, n, s));
   for (int i = 0; i < nshift; ++i) {
     CKM(launch_dw_copy(V.p[i], rhs, n, s));
@@ -268,11 +375,11 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
   }
   // One iteration: t = H_oe p; w = p - k^2 H_eo t with ||w||^2 = <p, Mhat^dag Mhat p>;
   // alpha; t = H^dag_oe w; the last hop forms Ap at its site and applies
-  // r -= alpha Ap with ||r||^2 (Ap is not stored); beta; then the x_i and p_i
-  // of every shift in one pass.
+  // r -= alpha Ap with ||r||^2 (Ap is not stored); beta; p = r + beta p.
   const double k2 = -P.kappa * P.kappa;
   float4 *t = G.vec_odd(G.vt), *w = G.vec_even(G.vw);
-  auto iteration = [&]() -> cudaError_t {
+  auto iteration = [&](int slot) -> cudaError_t {
+    float4 *r = ring[slot];
     HopParams H = G.hop_params(PREC_DW, 1, pb, nullptr, t, 0.0, 1.0, nullptr);
     H.guard = &S->halt;
     cudaError_t e = launch_hop(PREC_DW, H, false, false, false, s);
@@ -285,9 +392,9 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
     if (G.side) {
       if ((e = cudaEventRecord(G.ev_fork, s))) return e;
       if ((e = cudaStreamWaitEvent(G.side, G.ev_fork, 0))) return e;
-      if ((e = launch_ms_alpha(G.partials, nhop, S, G.side))) return e;
+      if ((e = launch_ms_alpha(G.partials, nhop, S, B, slot, G.side))) return e;
       if ((e = cudaEventRecord(G.ev_join, G.side))) return e;
-    } else if ((e = launch_ms_alpha(G.partials, nhop, S, s))) {
+    } else if ((e = launch_ms_alpha(G.partials, nhop, S, B, slot, s))) {
       return e;
     }
     H = G.hop_params(PREC_DW, 1, w, nullptr, t, 0.0, 1.0, nullptr);
@@ -296,11 +403,17 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
     if (G.side && (e = cudaStreamWaitEvent(s, G.ev_join, 0))) return e;
     H = G.hop_params(PREC_DW, 0, t, w, nullptr, 1.0, k2, G.partials);
     H.guard = &S->halt;
-    if ((e = launch_hop_dw_r(H, r, &S->alpha_dw, s))) return e;
-    return launch_ms_beta_xp(G.partials, nhop, nblas, S, V, r, pb, n, s);
+    if ((e = launch_hop_dw_r(H, r_last, r, &S->alpha_dw, s))) return e;
+    r_last = r;
+    return launch_ms_beta_p(G.partials, nhop, nblas, S, B, slot, r, pb, n, s);
   };
   for (;;) {
-    for (int k = 0; k < kMsCheckEvery; ++k) CKM(iteration());
+    for (int k = 0; k < kMsCheckEvery; ++k) {
+      const int slot = k % nring;
+      CKM(iteration(slot));
+      // (a poll ends a block too, so that x_i is final when the solve has halted)
+      if (slot + 1 == nring || k + 1 == kMsCheckEvery) CKM(launch_ms_steps(V, R, S, B, nblas, n, s));
+    }
     CKM(cudaMemcpyAsync(H, S, sizeof(MsScalars), cudaMemcpyDeviceToHost, s));
     CKM(cudaStreamSynchronize(s));
     if (P.verbose >= 3)
@@ -355,17 +468,23 @@ cudaError_t launch_ms_start(const double *partials, int n, MsScalars *S, double 
   return cudaGetLastError();
 }
 
-cudaError_t launch_ms_alpha(const double *partials, int nhop, MsScalars *S, cudaStream_t s) {
+cudaError_t launch_ms_alpha(const double *partials, int nhop, MsScalars *S, MsSteps *B, int slot, cudaStream_t s) {
   note_launch();
-  return launch_pdl(ms_alpha_kernel, 1, kReduceThreads, 0, s, partials, nhop, S);
+  return launch_pdl(ms_alpha_kernel, 1, kReduceThreads, 0, s, partials, nhop, S, B, slot);
 }
 
-cudaError_t launch_ms_beta_xp(const double *partials, int nhop, int nblas, MsScalars *S, const MsVectors &V,
-                              const float4 *r, float4 *pb, int64_t n, cudaStream_t s) {
+cudaError_t launch_ms_beta_p(const double *partials, int nhop, int nblas, MsScalars *S, MsSteps *B, int slot,
+                             const float4 *r, float4 *pb, int64_t n, cudaStream_t s) {
   note_launch(2);
-  const cudaError_t e = launch_pdl(ms_beta_kernel, 1, kReduceThreads, 0, s, partials, nhop, S);
+  const cudaError_t e = launch_pdl(ms_beta_kernel, 1, kReduceThreads, 0, s, partials, nhop, S, B, slot);
   if (e != cudaSuccess) return e;
-  return launch_pdl(ms_xp_kernel, nblas, kBlasThreads, 0, s, pb, r, V, n, S);
+  return launch_pdl(ms_p_kernel, nblas, kBlasThreads, 0, s, pb, r, n, S);
+}
+
+cudaError_t launch_ms_steps(const MsVectors &V, const MsResiduals &R, const MsScalars *S, const MsSteps *B, int nblas,
+                            int64_t n, cudaStream_t s) {
+  note_launch();
+  return launch_pdl(ms_steps_kernel, nblas, kBlasThreads, 0, s, V, R, n, S, B);
 }
 
 cudaError_t launch_ms_resid(const float4 *rhs, const float4 *Ax, const float4 *x, double sigma, int64_t n,

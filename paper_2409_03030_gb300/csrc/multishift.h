@@ -9,19 +9,32 @@
 namespace jqcd {
 
 constexpr int kMsMaxShifts = 32;
+constexpr int kMsBlock = 8;  // iterations between two updates of the shifted vectors
 
 // Device-resident scalars of one multi-shift solve.
 struct MsScalars {
   double rr, alpha, alpha_prev, beta, stop_rr, rhs2;
   double sigma[kMsMaxShifts], zeta_prev[kMsMaxShifts], zeta[kMsMaxShifts], zeta_next[kMsMaxShifts];
-  double alpha_s[kMsMaxShifts], beta_s[kMsMaxShifts], true_rr[kMsMaxShifts];
+  double alpha_s[kMsMaxShifts], true_rr[kMsMaxShifts];
   int active[kMsMaxShifts], conv_iter[kMsMaxShifts];
-  int xact[kMsMaxShifts];  // shifts whose x_i takes this iteration's update (active before beta)
   float2 alpha_dw;         // alpha as a (hi, lo) pair for the fused r update
   int nshift, iters, max_iters;
   int done;  // 1 every shift converged, 2 breakdown, 3 maxiter
   int halt;
-  int final_x;  // beta halted the solve: the x_i update of that iteration is still due
+};
+
+// The shifted updates of the iterations since the last pass over the shifts:
+// step j has x_i += alpha p_i (when xact) and p_i = zeta r_j + beta p_i (when
+// pact), with the coefficients as (hi, lo) pairs.
+struct MsSteps {
+  float2 alpha[kMsBlock][kMsMaxShifts], zeta[kMsBlock][kMsMaxShifts], beta[kMsBlock][kMsMaxShifts];
+  unsigned char xact[kMsBlock][kMsMaxShifts], pact[kMsBlock][kMsMaxShifts];
+  int n;  // steps recorded
+};
+
+// The residual r_j of each recorded step.
+struct MsResiduals {
+  const float4 *r[kMsBlock];
 };
 
 // Per-shift solution and search direction (even parity, double-word).
@@ -34,12 +47,16 @@ struct GaugeEntry;
 
 cudaError_t launch_ms_start(const double *partials, int n, MsScalars *S, double tol2, int max_iters,
                             cudaStream_t s);
-// alpha from the per-hop-block partials of ||Mhat p||^2.
-cudaError_t launch_ms_alpha(const double *partials, int nhop, MsScalars *S, cudaStream_t s);
-// beta from the per-hop-block partials of ||r||^2, then x_i += alpha_i p_i,
-// p = r + beta p and p_i = zeta_i r + beta_i p_i in one pass over the shifts.
-cudaError_t launch_ms_beta_xp(const double *partials, int nhop, int nblas, MsScalars *S, const MsVectors &V,
-                              const float4 *r, float4 *pb, int64_t n, cudaStream_t s);
+// alpha from the per-hop-block partials of ||Mhat p||^2; slot: this
+// iteration's place among the steps (0 starts a new record).
+cudaError_t launch_ms_alpha(const double *partials, int nhop, MsScalars *S, MsSteps *B, int slot, cudaStream_t s);
+// beta from the per-hop-block partials of ||r||^2 and the record of the
+// shifted updates (step slot), then p = r + beta p.
+cudaError_t launch_ms_beta_p(const double *partials, int nhop, int nblas, MsScalars *S, MsSteps *B, int slot,
+                             const float4 *r, float4 *pb, int64_t n, cudaStream_t s);
+// The recorded updates of every shift, in one pass over x_i and p_i.
+cudaError_t launch_ms_steps(const MsVectors &V, const MsResiduals &R, const MsScalars *S, const MsSteps *B, int nblas,
+                            int64_t n, cudaStream_t s);
 cudaError_t launch_ms_resid(const float4 *rhs, const float4 *Ax, const float4 *x, double sigma, int64_t n,
                             double *partials, int nblocks, cudaStream_t s);
 

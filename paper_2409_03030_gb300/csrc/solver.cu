@@ -30,6 +30,7 @@ constexpr int kMaxRestarts = 8;
 
 GaugeEntry::~GaugeEntry() {
   for (void *p : device_allocs) cudaFree(p);
+  drop_ms_ring();
   if (S_host) cudaFreeHost(S_host);
   if (ms_S_host) cudaFreeHost(ms_S_host);
   if (ev0) cudaEventDestroy(ev0);
@@ -42,6 +43,11 @@ GaugeEntry::~GaugeEntry() {
 cudaError_t GaugeEntry::alloc(void **p, size_t bytes) {
   *p = nullptr;
   cudaError_t e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
+  if (e == cudaErrorMemoryAllocation && !ms_r.empty()) {
+    cudaGetLastError();
+    drop_ms_ring();  // cudaFree waits for the device: nothing still reads them
+    e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
+  }
   if (e == cudaSuccess) device_allocs.push_back(*p);
   return e;
 }

@@ -38,7 +38,9 @@ struct GaugeEntry {
   double *lcanon = nullptr;
   // multi-shift CG workspace: per-shift search directions and scalars
   std::vector<float4 *> ms_p, ms_x;  // ms_x: solutions of the host-buffer entry
+  std::vector<float4 *> ms_r;        // residuals of a block of iterations, beside vr
   MsScalars *ms_S = nullptr;
+  MsSteps *ms_B = nullptr;
   MsScalars *ms_S_host = nullptr;  // pinned mirror
   // staggered workspace (double-word, whole lattice: even half then odd half)
   float4 *sb = nullptr, *sx = nullptr, *sr = nullptr, *sp = nullptr, *sAp = nullptr, *st = nullptr,
@@ -78,6 +80,8 @@ struct GaugeEntry {
   cudaError_t ensure_f64();
   cudaError_t ensure_force();
   cudaError_t ensure_multishift(int nshift);
+  void ensure_ms_ring();
+  void drop_ms_ring();
   cudaError_t ensure_staggered();
   cudaError_t ensure_hmc();
   // fermion-solve history of a trajectory: previous X, Y and two start vectors
@@ -106,10 +110,11 @@ cudaError_t apply_mdagm(const GaugeEntry &G, int prec, double kappa, const void 
 cudaError_t launch_hop_dw_cg(const HopParams &P, const float4 *p, float4 *x, float4 *r,
                              const SolverScalars *S, cudaStream_t s);
 
-// The same without x: Ap stays in registers, r -= alpha Ap with alpha =
-// *alpha_dw (device, hi/lo pair), P.partials gets ||r||^2 per hop block
-// (multi-shift CG, whose x_i are updated per shift elsewhere).
-cudaError_t launch_hop_dw_r(const HopParams &P, float4 *r, const float2 *alpha_dw, cudaStream_t s);
+// The same without x: Ap stays in registers, r = r_in - alpha Ap with alpha =
+// *alpha_dw (device, hi/lo pair; r may be r_in), P.partials gets ||r||^2 per
+// hop block (multi-shift CG, whose x_i are updated per shift elsewhere).
+cudaError_t launch_hop_dw_r(const HopParams &P, const float4 *r_in, float4 *r, const float2 *alpha_dw,
+                            cudaStream_t s);
 
 // The same for the inner CG of the mixed solver in hop precision prec (FP32 or
 // FP16 with norm): p, t and w in that precision, xs and rs FP32, alpha =

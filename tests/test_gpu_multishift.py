@@ -98,3 +98,23 @@ def test_multishift_full_size(jq):
     res = shifted_residual(dims, U, rhs, x3, 0.12, shifts[3])
     assert res <= 1e-10 * (1 + 1e-6) and abs(res - infos[3]["true_rel_resid"]) <= 1e-12
     g.free()
+
+
+@pytest.mark.parametrize("maxiter", [1, 7, 8, 9, 17])
+@pytest.mark.parametrize("nshift", [1, 5, 32])
+def test_multishift_block_edges(jq, nshift, maxiter):
+    """The shifted vectors are updated for several iterations at once: after any
+    number of iterations, at the ends of a block and inside one, every x_i is the
+    iterate of the plain CG on its own shifted system (bound as for the solves)."""
+    jqcd, ctx = jq
+    dims = (6, 4, 2, 8)
+    U = synth.gauge(dims, "expi", eps=0.3, seed=107)
+    rhs = oracle.zero_parity(dims, synth.gaussian_spinor(dims, seed=108), 1)
+    shifts = [0.0, 0.02, 0.3, 2.5, 40.0, *np.geomspace(1e-3, 1.0, 27)][:nshift]
+    g = ctx.gauge_upload(dims, U)
+    xs, infos, st = g.cg_multishift(rhs, 0.12, shifts, tol=1e-13, maxiter=maxiter, check=False)
+    assert st == jqcd.ENOCONV and infos[0]["iters"] == maxiter
+    for sigma, x in list(zip(shifts, xs))[:6]:
+        xo, *_ = oracle.cg_shift(dims, U, rhs, 0.12, sigma, eo=True, tol=1e-13, maxiter=maxiter)
+        assert rel(x, xo) <= 1e-9, sigma
+    g.free()
