@@ -22,8 +22,8 @@
 namespace jqcd {
 
 template <int MU, int PREC, bool DAG>
-__device__ __forceinline__ void hop_dir(const HopParams &P, int x, int y, int z, int t,
-                                        int64_t idx, typename PT<PREC>::C (&acc)[4][3]) {
+__device__ __forceinline__ void hop_dir(const HopParams &P, const HopSite &site,
+                                        typename PT<PREC>::C (&acc)[4][3]) {
   typedef PT<PREC> T;
   typedef typename T::C C;
   const Geom &g = P.g;
@@ -32,39 +32,23 @@ __device__ __forceinline__ void hop_dir(const HopParams &P, int x, int y, int z,
   const size_t link_bytes = (size_t)T::kLinkChunks * 16 * g.vh;  // one (parity, mu) block
   // forward neighbour x + mu: (1 - gamma_mu) U_mu(x) psi(x+mu)
   {
-    int xf = x, yf = y, zf = z, tf = t;
-    bool neg = false;
-    if (MU == 0) xf = (x + 1 == g.nx) ? 0 : x + 1;
-    if (MU == 1) yf = (y + 1 == g.ny) ? 0 : y + 1;
-    if (MU == 2) zf = (z + 1 == g.nz) ? 0 : z + 1;
-    if (MU == 3) {
-      if (t + 1 == g.nt) { tf = 0; neg = g.tanti != 0; } else tf = t + 1;
-    }
-    const int64_t nf = cb_index(g, xf, yf, zf, tf);
+    const unsigned off = hop_offset(g, site, 2 * MU);
     C psi[4][3], h[2][3], r[2][3], u[3][3];
-    T::load_spinor(P.in, g.vh, nf, psi);
+    T::load_spinor(P.in, g.vh, (off & ~1u) >> 4, psi);
     project<MU, DAG ? 1 : -1>(psi, h);
-    T::negate_if(h, neg);
-    T::load_link(gbase + link_bytes * (size_t)(p * 4 + MU), g.vh, idx, u);
+    T::negate_if(h, off & 1u);
+    T::load_link(gbase + link_bytes * (size_t)(p * 4 + MU), g.vh, site.idx, u);
     matvec2<false>(u, h, r);
     reconstruct<MU, DAG ? 1 : -1>(r, acc);
   }
   // backward neighbour x - mu: (1 + gamma_mu) U_mu(x-mu)^dag psi(x-mu)
   {
-    int xb = x, yb = y, zb = z, tb = t;
-    bool neg = false;
-    if (MU == 0) xb = (x == 0) ? g.nx - 1 : x - 1;
-    if (MU == 1) yb = (y == 0) ? g.ny - 1 : y - 1;
-    if (MU == 2) zb = (z == 0) ? g.nz - 1 : z - 1;
-    if (MU == 3) {
-      if (t == 0) { tb = g.nt - 1; neg = g.tanti != 0; } else tb = t - 1;
-    }
-    const int64_t nb = cb_index(g, xb, yb, zb, tb);
+    const unsigned off = hop_offset(g, site, 2 * MU + 1);
     C psi[4][3], h[2][3], r[2][3], u[3][3];
-    T::load_spinor(P.in, g.vh, nb, psi);
+    T::load_spinor(P.in, g.vh, (off & ~1u) >> 4, psi);
     project<MU, DAG ? -1 : 1>(psi, h);
-    T::negate_if(h, neg);
-    T::load_link(gbase + link_bytes * (size_t)((1 - p) * 4 + MU), g.vh, nb, u);
+    T::negate_if(h, off & 1u);
+    T::load_link(gbase + link_bytes * (size_t)((1 - p) * 4 + MU), g.vh, (off & ~1u) >> 4, u);
     matvec2<true>(u, h, r);
     reconstruct<MU, DAG ? -1 : 1>(r, acc);
   }
@@ -81,17 +65,16 @@ __global__ void __launch_bounds__(kHopThreads) hop_kernel(const HopParams P) {
   dwacc nrm{0.f, 0.f};
   double nrm64 = 0.0;  // FP64 hops accumulate their norm in FP64
   if (active) {
-    int x, y, z, t;
-    cb_coords(P.g, idx, P.out_parity, x, y, z, t);
+    const HopSite site = hop_site(P.g, (unsigned)idx, P.out_parity);
     C acc[4][3];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc[a][c] = T::zero();
-    hop_dir<0, PREC, DAG>(P, x, y, z, t, idx, acc);
-    hop_dir<1, PREC, DAG>(P, x, y, z, t, idx, acc);
-    hop_dir<2, PREC, DAG>(P, x, y, z, t, idx, acc);
-    hop_dir<3, PREC, DAG>(P, x, y, z, t, idx, acc);
+    hop_dir<0, PREC, DAG>(P, site, acc);
+    hop_dir<1, PREC, DAG>(P, site, acc);
+    hop_dir<2, PREC, DAG>(P, site, acc);
+    hop_dir<3, PREC, DAG>(P, site, acc);
     const typename T::Scalar b = T::scalar(P.b, P.b_split);
     C o[4][3];
     if (AXPY) {

@@ -34,10 +34,11 @@ constexpr int kForceOwnChunks = 24;  // X and Y of the thread's own site
 constexpr int kForceNbChunks = 12;   // the neighbour spinor of the next part
 constexpr size_t kForceSmem = (size_t)(kForceOwnChunks + kForceNbChunks) * kForceThreads * 16;  // 72 KB
 
-// Issue the copies of one double-word spinor of site i into a stage column.
-__device__ __forceinline__ void stage_spinor_force(float4 *st, const float4 *f, int64_t vh, int64_t i) {
+// Issue the copies of one double-word spinor (byte offset off) into a stage
+// column.
+__device__ __forceinline__ void stage_spinor_force(float4 *st, const float4 *f, int64_t vh, unsigned off) {
 #pragma unroll
-  for (int k = 0; k < 12; ++k) cp_async16(st + k * kForceThreads, f + k * vh + i, false);
+  for (int k = 0; k < 12; ++k) cp_async16(st + k * kForceThreads, chunk_at(f + k * vh, off), false);
 }
 
 // a + phase<PH> b for complex double-word pairs (PH: 0 -> 1, 1 -> i, 2 -> -1,
@@ -120,12 +121,13 @@ struct FieldPair {
 // previous direction) when the call starts; Y(x + mu) is copied in during
 // part 0 and X(x + mu + 1) during part 1, each as soon as the stage has been
 // read.
-__device__ __forceinline__ void force_link(const Geom &g, int p, int64_t cb, int x, int y, int z, int t, int mu,
-                                           const FieldPair &F, const float4 *own, float4 *nst,
+// own_off, nb_off, next_off: byte offsets of the site, of x + mu (bit 0: the
+// hop crosses an antiperiodic boundary) and of x + mu + 1.
+__device__ __forceinline__ void force_link(const Geom &g, int p, unsigned own_off, unsigned nb_off, unsigned next_off,
+                                           int mu, const FieldPair &F, const float4 *own, float4 *nst,
                                            const float4 *gauge, float2 two_kappa, float4 *out) {
   const int64_t vh = g.vh;
-  bool neg;
-  const int64_t nb = hop_neighbour(g, x, y, z, t, 2 * mu, neg);  // x + mu, parity 1-p
+  const bool neg = nb_off & 1u;
   const float4 *Xn = p ? F.xe : F.xo, *Yn = p ? F.ye : F.yo;
   constexpr f2 kLane0 = 0x0000000080000000ull;
   p2 M[3][3];
@@ -138,10 +140,9 @@ __device__ __forceinline__ void force_link(const Geom &g, int p, int64_t cb, int
 #pragma unroll
       for (int k = 0; k < 12; ++k) s4[k / 3][k % 3] = ld_p2(nst + k * kForceThreads);
       if (part == 0) {
-        stage_spinor_force(nst, Yn, vh, nb);
+        stage_spinor_force(nst, Yn, vh, nb_off & ~1u);
       } else if (mu < 3) {
-        bool neg1;
-        stage_spinor_force(nst, Xn, vh, hop_neighbour(g, x, y, z, t, 2 * mu + 2, neg1));
+        stage_spinor_force(nst, Xn, vh, next_off & ~1u);
       }
       cp_async_commit();
       if (part) adjoint_rt(mu, 1, s4, v);
@@ -199,10 +200,10 @@ __device__ __forceinline__ void force_link(const Geom &g, int p, int64_t cb, int
   }
   p2 U[3][3];
   {
-    const ulonglong2 *L = reinterpret_cast<const ulonglong2 *>(gauge) + (size_t)((p * 4 + mu) * 9) * vh + cb;
+    const ulonglong2 *L = reinterpret_cast<const ulonglong2 *>(gauge) + (size_t)((p * 4 + mu) * 9) * vh;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const ulonglong2 v = __ldcs(L + k * vh);
+      const ulonglong2 v = __ldcs(chunk_at(L + k * vh, own_off));
       U[k / 3][k % 3] = p2{v.x, v.y};
     }
   }
@@ -210,7 +211,7 @@ __device__ __forceinline__ void force_link(const Geom &g, int p, int64_t cb, int
   const float fs = neg ? -1.f : 1.f;  // boundary sign, exact
   const f2 fh = f2_make(fs * two_kappa.x, fs * two_kappa.x);
   const mul2 Fm{fh, f2_make(fs * two_kappa.y, fs * two_kappa.y)};
-  ulonglong2 *o = reinterpret_cast<ulonglong2 *>(out) + (size_t)((p * 4 + mu) * 9) * vh + cb;
+  const ulonglong2 *o = reinterpret_cast<ulonglong2 *>(out) + (size_t)((p * 4 + mu) * 9) * vh;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const p2 col[3] = {M[0][a], M[1][a], M[2][a]};
@@ -219,7 +220,7 @@ __device__ __forceinline__ void force_link(const Geom &g, int p, int64_t cb, int
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const p2 q = p2_norm(acc2_get(acc2_first(Fm, p2_norm(Gc[i]))));
-      __stcs(o + (3 * i + a) * vh, make_ulonglong2(q.h, q.l));
+      __stcs(const_cast<ulonglong2 *>(chunk_at(o + (3 * i + a) * vh, own_off)), make_ulonglong2(q.h, q.l));
     }
   }
 }
@@ -242,17 +243,21 @@ __global__ void __launch_bounds__(kForceThreads, 3) force_kernel(Geom g, FieldPa
   const float4 *Xh = p ? F.xo : F.xe, *Yh = p ? F.yo : F.ye;
   float4 *own = fsm + threadIdx.x;
   float4 *nst = fsm + kForceOwnChunks * kForceThreads + threadIdx.x;
-  int x, y, z, t;
-  cb_coords(g, cb, p, x, y, z, t);
-  stage_spinor_force(own, Xh, g.vh, cb);
-  stage_spinor_force(own + 12 * kForceThreads, Yh, g.vh, cb);
-  {
-    bool neg0;
-    stage_spinor_force(nst, p ? F.xe : F.xo, g.vh, hop_neighbour(g, x, y, z, t, 0, neg0));  // X(x + 0)
-  }
+  const HopSite site = hop_site(g, (unsigned)cb, p);
+  const unsigned own_off = 16u * (unsigned)cb;
+  stage_spinor_force(own, Xh, g.vh, own_off);
+  stage_spinor_force(own + 12 * kForceThreads, Yh, g.vh, own_off);
+  unsigned o0 = hop_offset(g, site, 0), o1 = hop_offset(g, site, 2), o2 = hop_offset(g, site, 4);
+  const unsigned o3 = hop_offset(g, site, 6);
+  stage_spinor_force(nst, p ? F.xe : F.xo, g.vh, o0 & ~1u);  // X(x + 0)
   cp_async_commit();
 #pragma unroll 1
-  for (int mu = 0; mu < 4; ++mu) force_link(g, p, cb, x, y, z, t, mu, F, own, nst, gauge, two_kappa, out);
+  for (int mu = 0; mu < 4; ++mu) {
+    force_link(g, p, own_off, o0, o1, mu, F, own, nst, gauge, two_kappa, out);
+    o0 = o1;
+    o1 = o2;
+    o2 = o3;
+  }
 }
 
 // out = gamma5 in on a whole-lattice double-word spinor (chunks k = 3*spin + c;
@@ -316,6 +321,7 @@ __global__ void linkfield_unpack_kernel(Geom g, const float4 *__restrict__ dwf, 
 cudaError_t launch_fermi_force(const Geom &g, const float4 *xe, const float4 *xo, const float4 *ye,
                                const float4 *yo, const float4 *gauge_dw, double kappa, float4 *out,
                                cudaStream_t s) {
+  if (g.vh >= kMaxHopSites) return cudaErrorInvalidValue;  // 32-bit offsets
   static bool configured = false;  // 72 KB of dynamic shared memory needs the opt-in
   if (!configured) {
     const cudaError_t e = cudaFuncSetAttribute(force_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

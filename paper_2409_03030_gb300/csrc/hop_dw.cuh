@@ -77,34 +77,56 @@ __device__ __forceinline__ int64_t hop_neighbour(const Geom &g, int x, int y, in
   return cb_index(g, x, y, z, t);
 }
 
-// Byte offsets (16 x checkerboard index) of the eight neighbours of site idx
-// of parity p, hop d = 2 mu + backward; bit 0 is set on a hop that crosses an
-// antiperiodic time boundary.  32-bit arithmetic throughout: a resident gauge
-// field takes 2688 bytes per site of one parity, so vh < 2^27 on any device
-// (launch_hop refuses more) and 16 idx < 2^31.  Each neighbour is one select
-// of a constant step; the 64-bit coordinates-to-index form took about 25
-// instructions per hop.
+// A site of one parity and its neighbours in 32-bit arithmetic: a resident
+// gauge field takes 2688 bytes per site of one parity, so vh < 2^27 on any
+// device (launch_hop and the other entries refuse more) and 16 idx < 2^31.
 constexpr int64_t kMaxHopSites = (int64_t)1 << 27;
-__device__ __forceinline__ void hop_offsets(const Geom &g, unsigned idx, int p, unsigned (&off)[8]) {
-  const unsigned nxh = g.nxh, ny = g.ny, nz = g.nz;
-  const unsigned xh = idx % nxh;
-  unsigned r = idx / nxh;
-  const unsigned y = r % ny;
-  r /= ny;
-  const unsigned z = r % nz;
-  const unsigned t = r / nz;
-  const bool odd = (y + z + t + p) & 1;  // x = 2 xh + odd
-  const unsigned sz = nxh * ny, st = sz * nz, vh = (unsigned)g.vh;
-  const unsigned neg = g.tanti ? 1u : 0u;
-  const bool tl = t + 1 == (unsigned)g.nt, tf = t == 0;
-  off[0] = 16u * (odd ? (xh + 1 == nxh ? idx + 1 - nxh : idx + 1) : idx);
-  off[1] = 16u * (odd ? idx : (xh == 0 ? idx + nxh - 1 : idx - 1));
-  off[2] = 16u * (y + 1 == ny ? idx + nxh - sz : idx + nxh);
-  off[3] = 16u * (y == 0 ? idx + sz - nxh : idx - nxh);
-  off[4] = 16u * (z + 1 == nz ? idx + sz - st : idx + sz);
-  off[5] = 16u * (z == 0 ? idx + st - sz : idx - sz);
-  off[6] = 16u * (tl ? idx + st - vh : idx + st) | (tl ? neg : 0u);
-  off[7] = 16u * (tf ? idx + vh - st : idx - st) | (tf ? neg : 0u);
+struct HopSite {
+  unsigned idx, xh, y, z, t;
+  bool odd;  // x = 2 xh + odd
+};
+__device__ __forceinline__ HopSite hop_site(const Geom &g, unsigned idx, int p) {
+  HopSite s;
+  s.idx = idx;
+  s.xh = idx % (unsigned)g.nxh;
+  unsigned r = idx / (unsigned)g.nxh;
+  s.y = r % (unsigned)g.ny;
+  r /= (unsigned)g.ny;
+  s.z = r % (unsigned)g.nz;
+  s.t = r / (unsigned)g.nz;
+  s.odd = (s.y + s.z + s.t + p) & 1;
+  return s;
+}
+
+// Byte offset (16 x checkerboard index) of the neighbour of hop d = 2 mu +
+// backward; bit 0 is set when the hop crosses an antiperiodic time boundary.
+// d is a constant where the hops are unrolled.  One select of a constant step
+// and one 32-bit offset beside grid-uniform chunk planes replace about 25
+// instructions of 64-bit coordinates-to-index arithmetic per hop and two per
+// chunk address.
+__device__ __forceinline__ unsigned hop_offset(const Geom &g, const HopSite &s, int d) {
+  const unsigned idx = s.idx, nxh = g.nxh, sz = nxh * (unsigned)g.ny, st = sz * (unsigned)g.nz;
+  switch (d) {
+    case 0: return 16u * (s.odd ? (s.xh + 1 == nxh ? idx + 1 - nxh : idx + 1) : idx);
+    case 1: return 16u * (s.odd ? idx : (s.xh == 0 ? idx + nxh - 1 : idx - 1));
+    case 2: return 16u * (s.y + 1 == (unsigned)g.ny ? idx + nxh - sz : idx + nxh);
+    case 3: return 16u * (s.y == 0 ? idx + sz - nxh : idx - nxh);
+    case 4: return 16u * (s.z + 1 == (unsigned)g.nz ? idx + sz - st : idx + sz);
+    case 5: return 16u * (s.z == 0 ? idx + st - sz : idx - sz);
+    case 6: {
+      const bool e = s.t + 1 == (unsigned)g.nt;
+      return 16u * (e ? idx + st - (unsigned)g.vh : idx + st) | (e && g.tanti ? 1u : 0u);
+    }
+    default: {
+      const bool e = s.t == 0;
+      return 16u * (e ? idx + (unsigned)g.vh - st : idx - st) | (e && g.tanti ? 1u : 0u);
+    }
+  }
+}
+
+// Address of the 16-byte chunk at byte offset off of a chunk plane.
+template <typename T> __device__ __forceinline__ const T *chunk_at(const T *plane, unsigned off) {
+  return reinterpret_cast<const T *>(reinterpret_cast<const char *>(plane) + off);
 }
 
 }  // namespace jqcd

@@ -68,7 +68,7 @@ constexpr size_t kDwp2Smem = dwp_smem(kDwp2Threads);
 template <int NT, bool L1>
 __device__ __forceinline__ void stage_hop_p(float4 *st, const float4 *in, int64_t vh, unsigned off) {
 #pragma unroll
-  for (int k = 0; k < 12; ++k) cp_async16(st + k * NT, reinterpret_cast<const char *>(in + k * vh) + off, L1);
+  for (int k = 0; k < 12; ++k) cp_async16(st + k * NT, chunk_at(in + k * vh, off), L1);
 }
 
 // Issue the copies of the link of hop d (mu = d/2, backward when d is odd)
@@ -82,7 +82,7 @@ __device__ __forceinline__ void stage_link_p(float4 *st, const float4 *gauge, in
   const float4 *L = gauge + (int64_t)(((bwd ? 1 - p : p) * 4 + (d >> 1)) * 9) * vh;
   const unsigned off = bwd ? nb : own;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) cp_async16(st + k * NT, reinterpret_cast<const char *>(L + k * vh) + off, false);
+  for (int k = 0; k < 9; ++k) cp_async16(st + k * NT, chunk_at(L + k * vh, off), false);
 }
 
 __device__ __forceinline__ p2 ld_p2(const float4 *p) {
@@ -271,7 +271,11 @@ __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, cons
   float4 *const lnk = spn + kDwpStageChunks * NT;    // and of the two link stages
   unsigned *const tab = reinterpret_cast<unsigned *>(dsm + (kDwpStageChunks + 2 * kDwpLinkChunks) * NT) + tid;
   unsigned off[8];
-  hop_offsets(g, idx, p, off);
+  {
+    const HopSite site = hop_site(g, idx, p);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) off[d] = hop_offset(g, site, d);
+  }
   if (DSTEP == 1) {
 #pragma unroll
     for (int d = 0; d < 8; ++d) tab[d * NT] = off[d];

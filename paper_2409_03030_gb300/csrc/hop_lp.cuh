@@ -48,29 +48,34 @@ __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 
-// Copies of hop d's neighbour spinor (site nb of the input parity) and link
-// (forward: U_mu(idx) of parity p; backward: U_mu(nb) of parity 1-p); the
-// link goes to chunk planes LK .. LK + 2 of the stage.
+// Copies of hop d's neighbour spinor (byte offset nb, see hop_offset) and link
+// (forward: U_mu(x) of parity p at byte offset own; backward: U_mu of the
+// neighbour, parity 1-p); the link goes to chunk planes LK .. LK + 2 of the
+// stage.
+template <int PREC>
+__device__ __forceinline__ void lp_stage_spinor(float4 *st, const void *in, int64_t vh, unsigned nb) {
+  const int tid = threadIdx.x;
+  const float4 *src = reinterpret_cast<const float4 *>(in);
+  constexpr int N = PREC == PREC_F32 ? 6 : 3;
+#pragma unroll
+  for (int k = 0; k < N; ++k) cp_async16(st + k * kHopThreads + tid, chunk_at(src + k * vh, nb), true);
+  if (PREC == PREC_F16N)
+    cp_async4(lp_norm_slot(st + 3 * kHopThreads, tid), chunk_at(reinterpret_cast<const float *>(src + 3 * vh), nb >> 2));
+}
+template <bool LINK_L1>
+__device__ __forceinline__ void lp_stage_link(float4 *st, const float4 *gauge, int64_t vh, int p, unsigned own, int d,
+                                              unsigned nb) {
+  const bool bwd = (d & 1) != 0;
+  const float4 *L = gauge + (int64_t)(((bwd ? 1 - p : p) * 4 + (d >> 1)) * 3) * vh;
+  const unsigned off = bwd ? nb : own;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) cp_async16(st + k * kHopThreads + threadIdx.x, chunk_at(L + k * vh, off), LINK_L1);
+}
 template <int PREC, bool LINK_L1, int LK = LpStage<PREC>::kSpin>
 __device__ __forceinline__ void lp_stage_issue(float4 *st, const void *in, const float4 *gauge,
-                                               int64_t vh, int p, int64_t idx, int d, int64_t nb) {
-  typedef LpStage<PREC> S;
-  const int tid = threadIdx.x;
-  if (PREC == PREC_F32) {
-    const float4 *src = reinterpret_cast<const float4 *>(in) + nb;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) cp_async16(st + k * kHopThreads + tid, src + k * vh, true);
-  } else {
-    const uint4 *src = reinterpret_cast<const uint4 *>(in);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) cp_async16(st + k * kHopThreads + tid, src + k * vh + nb, true);
-    cp_async4(lp_norm_slot(st + 3 * kHopThreads, tid), reinterpret_cast<const float *>(src + 3 * vh) + nb);
-  }
-  const int mu = d >> 1;
-  const bool bwd = (d & 1) != 0;
-  const float4 *L = gauge + (size_t)(((bwd ? 1 - p : p) * 4 + mu) * 3) * vh + (bwd ? nb : idx);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) cp_async16(st + (LK + k) * kHopThreads + tid, L + k * vh, LINK_L1);
+                                               int64_t vh, int p, unsigned own, int d, unsigned nb) {
+  lp_stage_spinor<PREC>(st, in, vh, nb);
+  lp_stage_link<LINK_L1>(st + LK * kHopThreads, gauge, vh, p, own, d, nb);
 }
 
 // Spinor and link of one stage slot (st already offset by the thread).  For
@@ -136,24 +141,23 @@ template <int PREC, bool DAG, bool LINK_L1, int C = LpStage<PREC>::kChunks, int 
 __device__ __forceinline__ void lp_hop_site(float4 *smem, const void *in, const float4 *gauge,
                                             const Geom &g, int p, int64_t idx, cf (&acc)[4][3]) {
   const int64_t vh = g.vh;
-  int x, y, z, t;
-  cb_coords(g, idx, p, x, y, z, t);
+  const HopSite site = hop_site(g, (unsigned)idx, p);
+  const unsigned own = 16u * (unsigned)idx;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[a][c] = cf{0.f, 0.f};
   const int tid = threadIdx.x;
-  bool neg_next;
-  int64_t nb = hop_neighbour(g, x, y, z, t, 0, neg_next);
-  lp_stage_issue<PREC, LINK_L1, LK>(smem, in, gauge, vh, p, idx, 0, nb);
+  unsigned nb = hop_offset(g, site, 0);
+  lp_stage_issue<PREC, LINK_L1, LK>(smem, in, gauge, vh, p, own, 0, nb & ~1u);
   cp_async_commit();
 #pragma unroll
   for (int d = 0; d < 8; ++d) {
-    const bool neg = neg_next;
+    const bool neg = nb & 1u;
     if (d < 7) {
-      nb = hop_neighbour(g, x, y, z, t, d + 1, neg_next);
-      lp_stage_issue<PREC, LINK_L1, LK>(smem + ((d + 1) & 1) * C * kHopThreads, in, gauge, vh, p, idx, d + 1,
-                                        nb);
+      nb = hop_offset(g, site, d + 1);
+      lp_stage_issue<PREC, LINK_L1, LK>(smem + ((d + 1) & 1) * C * kHopThreads, in, gauge, vh, p, own, d + 1,
+                                        nb & ~1u);
     }
     cp_async_commit();
     cp_async_wait1();  // this thread's copies of hop d have landed

@@ -42,35 +42,14 @@ template <int PH> __device__ __forceinline__ cp2 add_phase(cp2 a, cp2 b) {
   return cp2{f2_add(a.re, b.im), f2_sub(a.im, b.re)};
 }
 
-// Copies of one spinor of hop d's neighbour site nb into a stage slot.
-template <int PREC>
-__device__ __forceinline__ void lp2_issue_spinor(float4 *st, const void *in, int64_t vh, int64_t nb) {
-  const int tid = threadIdx.x;
-  if (PREC == PREC_F32) {
-    const float4 *src = reinterpret_cast<const float4 *>(in) + nb;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) cp_async16(st + k * kHopThreads + tid, src + k * vh, true);
-  } else {
-    const uint4 *src = reinterpret_cast<const uint4 *>(in);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) cp_async16(st + k * kHopThreads + tid, src + k * vh + nb, true);
-    cp_async4(lp_norm_slot(st + 3 * kHopThreads, tid), reinterpret_cast<const float *>(src + 3 * vh) + nb);
-  }
-}
-
 template <int PREC>
 __device__ __forceinline__ void lp2_issue(float4 *st, const void *in0, const void *in1,
-                                          const float4 *gauge, int64_t vh, int p, int64_t idx, int d,
-                                          int64_t nb) {
+                                          const float4 *gauge, int64_t vh, int p, unsigned own, int d,
+                                          unsigned nb) {
   typedef Lp2Stage<PREC> S;
-  lp2_issue_spinor<PREC>(st, in0, vh, nb);
-  lp2_issue_spinor<PREC>(st + S::kSpin * kHopThreads, in1, vh, nb);
-  const int tid = threadIdx.x;
-  const int mu = d >> 1;
-  const bool bwd = (d & 1) != 0;
-  const float4 *L = gauge + (size_t)(((bwd ? 1 - p : p) * 4 + mu) * 3) * vh + (bwd ? nb : idx);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) cp_async16(st + (2 * S::kSpin + k) * kHopThreads + tid, L + k * vh, true);
+  lp_stage_spinor<PREC>(st, in0, vh, nb);
+  lp_stage_spinor<PREC>(st + S::kSpin * kHopThreads, in1, vh, nb);
+  lp_stage_link<true>(st + 2 * S::kSpin * kHopThreads, gauge, vh, p, own, d, nb);
 }
 
 // The two spinors of a stage slot (st offset by the thread) as packed
@@ -182,23 +161,22 @@ __device__ __forceinline__ void lp2_hop_site(float4 *smem, const void *in0, cons
   constexpr int C = Lp2Stage<PREC>::kChunks;
   constexpr int K = Lp2Stage<PREC>::kSpin;
   const int64_t vh = g.vh;
-  int x, y, z, t;
-  cb_coords(g, idx, p, x, y, z, t);
+  const HopSite site = hop_site(g, (unsigned)idx, p);
+  const unsigned own = 16u * (unsigned)idx;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[a][c] = cp2{0ull, 0ull};
   const int tid = threadIdx.x;
-  bool neg_next;
-  int64_t nb = hop_neighbour(g, x, y, z, t, 0, neg_next);
-  lp2_issue<PREC>(smem, in0, in1, gauge, vh, p, idx, 0, nb);
+  unsigned nb = hop_offset(g, site, 0);
+  lp2_issue<PREC>(smem, in0, in1, gauge, vh, p, own, 0, nb & ~1u);
   cp_async_commit();
 #pragma unroll
   for (int d = 0; d < 8; ++d) {
-    const bool neg = neg_next;
+    const bool neg = nb & 1u;
     if (d < 7) {
-      nb = hop_neighbour(g, x, y, z, t, d + 1, neg_next);
-      lp2_issue<PREC>(smem + ((d + 1) & 1) * C * kHopThreads, in0, in1, gauge, vh, p, idx, d + 1, nb);
+      nb = hop_offset(g, site, d + 1);
+      lp2_issue<PREC>(smem + ((d + 1) & 1) * C * kHopThreads, in0, in1, gauge, vh, p, own, d + 1, nb & ~1u);
     }
     cp_async_commit();
     cp_async_wait1();  // this thread's copies of hop d have landed
