@@ -105,9 +105,14 @@ __global__ void __launch_bounds__(kHopThreads) hop_kernel(const HopParams P) {
 }
 
 // Low-precision hop with the next hop's neighbour and link prefetched into
-// shared memory (hop_lp.cuh); same epilogue as hop_kernel.
+// shared memory (hop_lp.cuh); same epilogue as hop_kernel.  HBM-bound (78.6 us
+// = 6.5 TB/s at 32^3x64); six blocks per SM (84 registers) measured best:
+// 27.9 us at 24^3x48 against 28.2 us with the compiler's 72-80 registers, 28.8
+// us cut for seven; mixed FP16 solve 14.11 -> 13.94 ms, at 32^3x64 40.0 ->
+// 39.6 ms.  Plain loads (hop_kernel) ran 25.6 us at 24^3x48 but 83.2 us at
+// 32^3x64 and 4.9 against 3.9 us at 16^4.
 template <int PREC, bool DAG, bool AXPY, bool NORM>
-__global__ void __launch_bounds__(kHopThreads) hop_lp_kernel(const HopParams P) {
+__global__ void __launch_bounds__(kHopThreads, 6) hop_lp_kernel(const HopParams P) {
   typedef PT<PREC> T;
   extern __shared__ float4 lsm[];
   pdl_enter();

@@ -130,9 +130,10 @@ __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
 // Low-precision form for the inner CG: Ap = a w + b H^dag t in FP32 registers
 // (never rounded to the storage precision), then the FP32 update of the
 // inner solution xs and residual rs with alpha_f, as the unfused update
-// kernel does, and ||rs||^2 per hop block.
+// kernel does, and ||rs||^2 per hop block.  Cut for five blocks per SM (six
+// cost the FP16 solve 1.5% at 24^3x48).
 template <int PREC>
-__global__ void __launch_bounds__(kHopThreads)
+__global__ void __launch_bounds__(kHopThreads, 5)
     hop_lp_cg_kernel(const HopParams P, const void *__restrict__ p, float4 *__restrict__ xs,
                      float4 *__restrict__ rs, const SolverScalars *__restrict__ S) {
   typedef PT<PREC> T;
