@@ -52,13 +52,14 @@ __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
 // (forward: U_mu(x) of parity p at byte offset own; backward: U_mu of the
 // neighbour, parity 1-p); the link goes to chunk planes LK .. LK + 2 of the
 // stage.
-template <int PREC>
+// L1: the spinor through L1 or past it.
+template <int PREC, bool L1 = true>
 __device__ __forceinline__ void lp_stage_spinor(float4 *st, const void *in, int64_t vh, unsigned nb) {
   const int tid = threadIdx.x;
   const float4 *src = reinterpret_cast<const float4 *>(in);
   constexpr int N = PREC == PREC_F32 ? 6 : 3;
 #pragma unroll
-  for (int k = 0; k < N; ++k) cp_async16(st + k * kHopThreads + tid, chunk_at(src + k * vh, nb), true);
+  for (int k = 0; k < N; ++k) cp_async16(st + k * kHopThreads + tid, chunk_at(src + k * vh, nb), L1);
   if (PREC == PREC_F16N)
     cp_async4(lp_norm_slot(st + 3 * kHopThreads, tid), chunk_at(reinterpret_cast<const float *>(src + 3 * vh), nb >> 2));
 }

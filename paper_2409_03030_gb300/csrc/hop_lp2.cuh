@@ -11,7 +11,11 @@
 // Staging follows hop_lp.cuh: the next hop's two neighbour spinors and its
 // link are copied into shared memory with cp.async while the current hop
 // computes (two stages, chunk-major [chunk][thread], each thread touching
-// only its own column).
+// only its own column).  The copies go past L1: four blocks' stages leave it
+// about 50 KB, less than the bytes in flight, so allocating there limited
+// them (iteration graphs of the 24-solve batch, FP16 inner 135.6 -> 130.4 ms,
+// FP32 172.8 -> 156.7 ms of device time; loads straight into registers
+// instead of staged ones took 141 and 171-186 ms).
 #pragma once
 #include "dw2.cuh"
 #include "hop_lp.cuh"
@@ -47,9 +51,9 @@ __device__ __forceinline__ void lp2_issue(float4 *st, const void *in0, const voi
                                           const float4 *gauge, int64_t vh, int p, unsigned own, int d,
                                           unsigned nb) {
   typedef Lp2Stage<PREC> S;
-  lp_stage_spinor<PREC>(st, in0, vh, nb);
-  lp_stage_spinor<PREC>(st + S::kSpin * kHopThreads, in1, vh, nb);
-  lp_stage_link<true>(st + 2 * S::kSpin * kHopThreads, gauge, vh, p, own, d, nb);
+  lp_stage_spinor<PREC, false>(st, in0, vh, nb);
+  lp_stage_spinor<PREC, false>(st + S::kSpin * kHopThreads, in1, vh, nb);
+  lp_stage_link<false>(st + 2 * S::kSpin * kHopThreads, gauge, vh, p, own, d, nb);
 }
 
 // The two spinors of a stage slot (st offset by the thread) as packed
