@@ -1163,10 +1163,11 @@ jqcd_status jqcd_hmc_trajectory(jqcd_ctx *ctx, uint64_t gauge_id, const jqcd_hmc
     if (!e && nhist >= 1) e = launch_dw_copy(G->hXp, G->fX, nfull, s);
     return e;
   };
-  // leapfrog
   const double dt = hp->tau / hp->n_md;
+  // leapfrog; the half link steps that end one step and begin the next use the
+  // same momenta and are taken as one
+  CK(hmc_links_update(*G, 0.5 * dt, s), "link update");
   for (int step = 0; step < hp->n_md; ++step) {
-    CK(hmc_links_update(*G, 0.5 * dt, s), "link update");
     CK(hmc_gauge_force(*G, hp->beta, s), "gauge force");
     if (hp->fermions) {
       jqcd_solve_info fi;
@@ -1181,7 +1182,7 @@ jqcd_status jqcd_hmc_trajectory(jqcd_ctx *ctx, uint64_t gauge_id, const jqcd_hmc
                             G->fout, s), "fermion force");
     }
     CK(hmc_momenta_update(*G, hp->fermions ? G->fout : nullptr, 0.5 * dt, s), "momenta update");
-    CK(hmc_links_update(*G, 0.5 * dt, s), "link update");
+    CK(hmc_links_update(*G, step + 1 < hp->n_md ? dt : 0.5 * dt, s), "link update");
   }
   if (st == JQCD_OK) {
     S_f = 0.0;

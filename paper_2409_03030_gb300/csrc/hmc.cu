@@ -303,77 +303,125 @@ __global__ void mom_update_kernel(Geom g, double2 *__restrict__ P, const double2
   m3_store(P, g.vh, p, mu, cb, A);
 }
 
-// exp(X) for a 3x3 complex X with |X|_F <= 1, by the Cayley-Hamilton identity
-// X^3 = t X^2 - s X + d (t = tr X, s = ((tr X)^2 - tr X^2)/2, d = det X):
-// X^n = a_n + b_n X + c_n X^2 with a_{n+1} = d c_n, b_{n+1} = a_n - s c_n,
-// c_{n+1} = b_n + t c_n, so exp X = F0 + F1 X + F2 X^2 with
-// F = sum_n (a_n, b_n, c_n) / n!.  One matrix product (X^2) replaces the
-// products of a matrix Taylor series; the F are divided differences of exp
-// on the spectrum, smooth also for degenerate eigenvalues, and 18 terms
-// reach double precision for |X|_F <= 1 (checked against a dense matrix
-// exponential, degenerate spectra and a small trace included).  The count
-// of terms is fixed by nu >= |X|_F: the series' remainder after N terms is at
-// most nu^(N+1) / (N+1)! / (1 - nu / (N+2)), below 1e-17 for N = 10, 12, 15,
-// 18 at nu <= 1/8, 1/4, 1/2, 1 (a leapfrog step's eps P has |eps P|_F of
-// about 0.1; the 16^4 trajectory went 0.0649 -> 0.0634 s against 18 terms
-// always).  A count fixed per call measured faster than stopping at the
-// first negligible term.
-__device__ __forceinline__ m3 m3_exp(const m3 &X, double nu) {
+// exp(iQ) for a Hermitian 3x3 Q with |Q|_F <= 1, by the Cayley-Hamilton
+// identity Q^3 = t Q^2 - s Q + d (t = tr Q, s = ((tr Q)^2 - tr Q^2)/2, d = det Q,
+// all real): Q^n = a_n + b_n Q + c_n Q^2 with the real recurrence a_{n+1} =
+// d c_n, b_{n+1} = a_n - s c_n, c_{n+1} = b_n + t c_n, so exp(iQ) = F0 + F1 Q +
+// F2 Q^2 with F = sum_n i^n (a_n, b_n, c_n) / n!.  The F are divided
+// differences of exp on the spectrum, smooth also for degenerate eigenvalues,
+// and 18 terms reach double precision for |Q|_F <= 1.  The count of terms is
+// fixed by nu >= |Q|_F: the series' remainder after N terms is at most
+// nu^(N+1) / (N+1)! / (1 - nu / (N+2)), below 1e-17 for N = 10, 12, 15, 18 at nu
+// <= 1/8, 1/4, 1/2, 1.  A count fixed per call measured faster than stopping
+// at the first negligible term.  The kernel is bound by the FP64 pipe: a real
+// recurrence, the six independent entries of Q^2 and the real diagonal take
+// about 200 FP64 operations against 560 for a general complex matrix (link
+// update at 16^4 417 -> 209 us, the refresh of the link copies included).
+struct Herm3 {  // Q_ab for a <= b; Q_ba = conj(Q_ab)
+  double d0, d1, d2;
+  double2 e01, e02, e12;
+};
+
+__device__ __forceinline__ double abs2(double2 a) { return fma(a.x, a.x, a.y * a.y); }
+
+// f0 [diagonal] + f1 q + f2 s for complex f and real (diagonal) q, s
+__device__ __forceinline__ double2 comb_diag(double2 f0, double2 f1, double2 f2, double q, double s) {
+  return make_double2(fma(f2.x, s, fma(f1.x, q, f0.x)), fma(f2.y, s, fma(f1.y, q, f0.y)));
+}
+// f1 q + f2 s, and with conjugated q and s
+__device__ __forceinline__ double2 comb(double2 f1, double2 f2, double2 q, double2 s) {
+  return make_double2(fma(-f2.y, s.y, fma(f2.x, s.x, fma(-f1.y, q.y, f1.x * q.x))),
+                      fma(f2.y, s.x, fma(f2.x, s.y, fma(f1.y, q.x, f1.x * q.y))));
+}
+__device__ __forceinline__ double2 conj_d(double2 a) { return make_double2(a.x, -a.y); }
+
+__device__ __forceinline__ m3 m3_exp_i(const Herm3 &q, double nu) {
   const int nterms = nu <= 0.125 ? 10 : (nu <= 0.25 ? 12 : (nu <= 0.5 ? 15 : 18));
-  const m3 X2 = m3_mul(X, X);
-  const double2 t = cadd_d(cadd_d(X.e[0][0], X.e[1][1]), X.e[2][2]);
-  const double2 tr2 = cadd_d(cadd_d(X2.e[0][0], X2.e[1][1]), X2.e[2][2]);
-  const double2 tt = cmul_d(t, t);
-  const double2 sI = make_double2(0.5 * (tt.x - tr2.x), 0.5 * (tt.y - tr2.y));
-  const double2 m0 = cadd_d(cmul_d(X.e[1][1], X.e[2][2]), cmul_d(make_double2(-X.e[1][2].x, -X.e[1][2].y), X.e[2][1]));
-  const double2 m1 = cadd_d(cmul_d(X.e[1][0], X.e[2][2]), cmul_d(make_double2(-X.e[1][2].x, -X.e[1][2].y), X.e[2][0]));
-  const double2 m2 = cadd_d(cmul_d(X.e[1][0], X.e[2][1]), cmul_d(make_double2(-X.e[1][1].x, -X.e[1][1].y), X.e[2][0]));
-  const double2 d0 = cmul_d(X.e[0][0], m0), d1 = cmul_d(X.e[0][1], m1), d2 = cmul_d(X.e[0][2], m2);
-  const double2 d = make_double2(d0.x - d1.x + d2.x, d0.y - d1.y + d2.y);
-  double2 a = make_double2(1.0, 0.0), b = make_double2(0.0, 0.0), c = b;
-  double2 F0 = a, F1 = b, F2 = b;
+  const double n01 = abs2(q.e01), n02 = abs2(q.e02), n12 = abs2(q.e12);
+  Herm3 s;  // Q^2
+  s.d0 = fma(q.d0, q.d0, n01 + n02);
+  s.d1 = fma(q.d1, q.d1, n01 + n12);
+  s.d2 = fma(q.d2, q.d2, n02 + n12);
+  const double2 z01 = cmul_d(q.e02, conj_d(q.e12)), z02 = cmul_d(q.e01, q.e12), z12 = cmul_d(conj_d(q.e01), q.e02);
+  s.e01 = make_double2(fma(q.d0 + q.d1, q.e01.x, z01.x), fma(q.d0 + q.d1, q.e01.y, z01.y));
+  s.e02 = make_double2(fma(q.d0 + q.d2, q.e02.x, z02.x), fma(q.d0 + q.d2, q.e02.y, z02.y));
+  s.e12 = make_double2(fma(q.d1 + q.d2, q.e12.x, z12.x), fma(q.d1 + q.d2, q.e12.y, z12.y));
+  const double t = q.d0 + q.d1 + q.d2;
+  const double sI = 0.5 * (t * t - (s.d0 + s.d1 + s.d2));
+  // det Q = q00 (q11 q22 - |q12|^2) - q11 |q02|^2 - q22 |q01|^2 + 2 Re(q01 q12 conj(q02))
+  const double d = fma(q.d0, fma(q.d1, q.d2, -n12), -fma(q.d1, n02, q.d2 * n01)) +
+                   2.0 * fma(z02.x, q.e02.x, z02.y * q.e02.y);
+  double a = 1.0, b = 0.0, c = 0.0;
+  double2 F0 = make_double2(1.0, 0.0), F1 = make_double2(0.0, 0.0), F2 = F1;
 #pragma unroll
   for (int n = 1; n <= 18; ++n) {
     if (n > nterms) break;
-    const double inv = 1.0 / n;
-    const double2 dc = cmul_d(d, c), sc = cmul_d(sI, c), tc = cmul_d(t, c);
-    const double2 na = make_double2(dc.x * inv, dc.y * inv);
-    const double2 nb = make_double2((a.x - sc.x) * inv, (a.y - sc.y) * inv);
-    const double2 nc = make_double2((b.x + tc.x) * inv, (b.y + tc.y) * inv);
+    constexpr double kInv[19] = {0.0,      1.0,      1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,
+                                 1.0 / 7,  1.0 / 8,  1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13,
+                                 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18};
+    const double na = d * c * kInv[n], nb = fma(-sI, c, a) * kInv[n], nc = fma(t, c, b) * kInv[n];
     a = na;
     b = nb;
     c = nc;
-    F0 = cadd_d(F0, a);
-    F1 = cadd_d(F1, b);
-    F2 = cadd_d(F2, c);
+    if (n & 1) {  // i^n = i, -i
+      F0.y = n & 2 ? F0.y - a : F0.y + a;
+      F1.y = n & 2 ? F1.y - b : F1.y + b;
+      F2.y = n & 2 ? F2.y - c : F2.y + c;
+    } else {
+      F0.x = n & 2 ? F0.x - a : F0.x + a;
+      F1.x = n & 2 ? F1.x - b : F1.x + b;
+      F2.x = n & 2 ? F2.x - c : F2.x + c;
+    }
   }
   m3 E;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      double2 v = cadd_d(cmul_d(F1, X.e[i][j]), cmul_d(F2, X2.e[i][j]));
-      if (i == j) v = cadd_d(v, F0);
-      E.e[i][j] = v;
-    }
+  E.e[0][0] = comb_diag(F0, F1, F2, q.d0, s.d0);
+  E.e[1][1] = comb_diag(F0, F1, F2, q.d1, s.d1);
+  E.e[2][2] = comb_diag(F0, F1, F2, q.d2, s.d2);
+  E.e[0][1] = comb(F1, F2, q.e01, s.e01);
+  E.e[1][0] = comb(F1, F2, conj_d(q.e01), conj_d(s.e01));
+  E.e[0][2] = comb(F1, F2, q.e02, s.e02);
+  E.e[2][0] = comb(F1, F2, conj_d(q.e02), conj_d(s.e02));
+  E.e[1][2] = comb(F1, F2, q.e12, s.e12);
+  E.e[2][1] = comb(F1, F2, conj_d(q.e12), conj_d(s.e12));
   return E;
 }
 
-// U <- exp(eps P) U: exp(eps P / 2^k) with |eps P / 2^k|_F <= 1 by m3_exp,
-// squared k times (k = 0 for the step sizes of a trajectory)
-__global__ void exp_update_kernel(Geom g, double2 *__restrict__ U, const double2 *__restrict__ P, double eps) {
+// The double-word and 12-real FP32 copies of a link (same per-link layout as gauge_pack).
+__device__ __forceinline__ void link_copies(const m3 &A, int64_t blk, int64_t vh, int64_t cb, float4 *dwo,
+                                            float4 *f32o) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const double2 v = A.e[k / 3][k % 3];
+    const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
+    dwo[(blk * 9 + k) * vh + cb] =
+        make_float4(rh, ih, __double2float_rn(v.x - (double)rh), __double2float_rn(v.y - (double)ih));
+  }
+  const double2 e[6] = {A.e[0][0], A.e[0][1], A.e[0][2], A.e[1][0], A.e[1][1], A.e[1][2]};
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    f32o[(blk * 3 + j) * vh + cb] = make_float4((float)e[2 * j].x, (float)e[2 * j].y, (float)e[2 * j + 1].x,
+                                                (float)e[2 * j + 1].y);
+}
+
+// U <- exp(eps P) U and its double-word and FP32 copies.  P is anti-Hermitian
+// to the bit (momenta are set and updated with both halves of each pair alike),
+// so eps P = iQ with Q from its upper triangle; exp(iQ / 2^k) with |Q / 2^k|_F
+// <= 1 by m3_exp_i, squared k times (k = 0 for the step sizes of a trajectory).
+__global__ void exp_update_kernel(Geom g, double2 *__restrict__ U, const double2 *__restrict__ P, double eps,
+                                  float4 *__restrict__ dwo, float4 *__restrict__ f32o) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= 8 * g.vh) return;
   const int mu = (int)(q / (2 * g.vh));
   const int64_t r = q % (2 * g.vh);
   const int p = (int)(r / g.vh);
   const int64_t cb = r - (int64_t)p * g.vh;
-  m3 A = m3_load(P, g.vh, p, mu, cb);
-  double nrm = 0.0;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) nrm += A.e[a][b].x * A.e[a][b].x + A.e[a][b].y * A.e[a][b].y;
+  const double2 *Pl = P + (size_t)((p * 4 + mu) * 9) * g.vh + cb;
+  const double2 p01 = Pl[g.vh], p02 = Pl[2 * g.vh], p12 = Pl[5 * g.vh];
+  Herm3 h;  // Q = -i eps P: Q_ab = eps (P_ab.im, -P_ab.re)
+  h.d0 = Pl[0].y;
+  h.d1 = Pl[4 * g.vh].y;
+  h.d2 = Pl[8 * g.vh].y;
+  double nrm = h.d0 * h.d0 + h.d1 * h.d1 + h.d2 * h.d2 + 2.0 * (abs2(p01) + abs2(p02) + abs2(p12));
   nrm = fabs(eps) * sqrt(nrm);  // Frobenius norm of eps P
   int k = 0;
   double sc = eps;
@@ -382,13 +430,17 @@ __global__ void exp_update_kernel(Geom g, double2 *__restrict__ U, const double2
     sc *= 0.5;
     ++k;
   }
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) A.e[a][b] = make_double2(sc * A.e[a][b].x, sc * A.e[a][b].y);
-  m3 E = m3_exp(A, nrm);
+  h.d0 *= sc;
+  h.d1 *= sc;
+  h.d2 *= sc;
+  h.e01 = make_double2(sc * p01.y, -sc * p01.x);
+  h.e02 = make_double2(sc * p02.y, -sc * p02.x);
+  h.e12 = make_double2(sc * p12.y, -sc * p12.x);
+  m3 E = m3_exp_i(h, nrm);
   for (int i = 0; i < k; ++i) E = m3_mul(E, E);
-  m3_store(U, g.vh, p, mu, cb, m3_mul(E, m3_load(U, g.vh, p, mu, cb)));
+  const m3 V = m3_mul(E, m3_load(U, g.vh, p, mu, cb));
+  m3_store(U, g.vh, p, mu, cb, V);
+  link_copies(V, (int64_t)(p * 4 + mu), g.vh, cb, dwo, f32o);
 }
 
 // FP64 links -> double-word and 12-real FP32 copies (same per-link layout as gauge_pack)
@@ -400,20 +452,7 @@ __global__ void links_refresh_kernel(Geom g, const double2 *__restrict__ U, floa
   const int64_t r = q % (2 * g.vh);
   const int p = (int)(r / g.vh);
   const int64_t cb = r - (int64_t)p * g.vh;
-  const m3 A = m3_load(U, g.vh, p, mu, cb);
-  const int64_t blk = (int64_t)(p * 4 + mu);
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    const double2 v = A.e[k / 3][k % 3];
-    const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
-    dwo[(blk * 9 + k) * g.vh + cb] =
-        make_float4(rh, ih, __double2float_rn(v.x - (double)rh), __double2float_rn(v.y - (double)ih));
-  }
-  const double2 e[6] = {A.e[0][0], A.e[0][1], A.e[0][2], A.e[1][0], A.e[1][1], A.e[1][2]};
-#pragma unroll
-  for (int j = 0; j < 3; ++j)
-    f32o[(blk * 3 + j) * g.vh + cb] = make_float4((float)e[2 * j].x, (float)e[2 * j].y, (float)e[2 * j + 1].x,
-                                                  (float)e[2 * j + 1].y);
+  link_copies(m3_load(U, g.vh, p, mu, cb), (int64_t)(p * 4 + mu), g.vh, cb, dwo, f32o);
 }
 
 // FP64 link field -> canonical host layout a + 3(b + 3(site + V mu))
@@ -545,10 +584,9 @@ cudaError_t hmc_momenta_update(GaugeEntry &G, const float4 *Gf, double coef, cud
 
 cudaError_t hmc_links_update(GaugeEntry &G, double eps, cudaStream_t s) {
   note_launch();
-  exp_update_kernel<<<link_blocks(G.g.vh), kHmcThreads, 0, s>>>(G.g, (double2 *)G.gauge_f64, G.hP, eps);
-  cudaError_t e = cudaGetLastError();
-  if (!e) e = launch_hmc_links_refresh(G, s);
-  return e;
+  exp_update_kernel<<<link_blocks(G.g.vh), kHmcThreads, 0, s>>>(G.g, (double2 *)G.gauge_f64, G.hP, eps,
+                                                                (float4 *)G.gauge_dw, (float4 *)G.gauge_f32);
+  return cudaGetLastError();
 }
 
 }  // namespace jqcd

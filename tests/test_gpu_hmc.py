@@ -100,3 +100,22 @@ def test_second_order_energy_error(jq, fermions):
         dH.append(abs(info["dH"]))
         g.free()
     assert 2.8 < dH[0] / dH[1] < 5.5, dH
+
+
+@pytest.mark.parametrize("n_md", [1, 3])
+@pytest.mark.parametrize("tau", [0.02, 0.15, 0.35, 0.9, 3.0, 40.0])
+def test_link_update_exponential(jq, tau, n_md):
+    """With beta = 0 there is no force and a trajectory is exp(tau P) U: every
+    length of the exponential's series and its squarings.  Bound: FP64 rounding
+    of the series and two products (1e-14 relative), doubled by each squaring
+    (|tau P| of them, up to 8 tau)."""
+    jqcd, ctx = jq
+    dims = (4, 2, 6, 4)
+    U = synth.gauge(dims, "haar", seed=181)
+    normals = normals_for(dims, 182)
+    g = ctx.gauge_upload(dims, U)
+    info, st = g.hmc_trajectory(normals, None, 0.0, 0.0, tau=tau, n_md=n_md)
+    assert st == 0 and info["accepted"] == 1
+    want = oracle.exp_update(U, oracle.momenta(normals), tau)
+    assert rel(g.download(), want) <= 2e-15 * (10 + 8 * tau)
+    g.free()
