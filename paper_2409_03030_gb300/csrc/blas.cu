@@ -113,11 +113,11 @@ __global__ void finalize_sum_kernel(const double *partials, int n, double *out) 
   if (threadIdx.x == 0) *out = s;
 }
 
-__global__ void cg_alpha_kernel(const double *partials, int n, SolverScalars *S) {
+__global__ void cg_alpha_kernel(const double *partials, int n, SolverScalars *S, int x_code) {
   pdl_enter();
   if (S->halt) return;
   const double pAp = block_sum_partials(partials, n);
-  if (threadIdx.x == 0) cg_alpha_step(pAp, S);
+  if (threadIdx.x == 0) cg_alpha_step(pAp, S, x_code);
 }
 
 __global__ void cg_beta_kernel(const double *partials, int n, SolverScalars *S) {
@@ -180,9 +180,9 @@ cudaError_t launch_dw_xpay(float4 *p, const float4 *r, int64_t n, const SolverSc
   note_launch();
   return launch_pdl(dw_xpay_kernel, blas_blocks(n), kBlasThreads, 0, s, p, r, n, S);
 }
-cudaError_t launch_cg_alpha(const double *partials, int n, SolverScalars *S, cudaStream_t s) {
+cudaError_t launch_cg_alpha(const double *partials, int n, SolverScalars *S, cudaStream_t s, int x_code) {
   note_launch();
-  return launch_pdl(cg_alpha_kernel, 1, kReduceThreads, 0, s, partials, n, S);
+  return launch_pdl(cg_alpha_kernel, 1, kReduceThreads, 0, s, partials, n, S, x_code);
 }
 cudaError_t launch_cg_beta(const double *partials, int n, SolverScalars *S, cudaStream_t s) {
   note_launch();

@@ -28,7 +28,7 @@ __device__ __forceinline__ void store_f32(float4 *base, int64_t vh, int64_t i, c
 }
 
 template <int PREC>
-__global__ void mixed_xpay_kernel(void *__restrict__ p, const float4 *__restrict__ rs, int64_t vh,
+__global__ void mixed_xpay_kernel(void *p_out, const void *p, const float4 *__restrict__ rs, int64_t vh,
                                   const SolverScalars *S) {
   pdl_enter();
   if (S->halt) return;
@@ -45,7 +45,47 @@ __global__ void mixed_xpay_kernel(void *__restrict__ p, const float4 *__restrict
     q.re = fmaf(b, q.re, r.re);
     q.im = fmaf(b, q.im, r.im);
   }
-  PT<PREC>::store_spinor(p, vh, i, pv);
+  PT<PREC>::store_spinor(p_out, vh, i, pv);
+}
+
+// x_s is not needed while the inner loop iterates, so it is brought up to
+// date once per block of iterations from the directions they kept: per site
+// 8 x 52 + 192 bytes (FP16) instead of 8 x (52 + 192) in the fused last hops,
+// which are bound by HBM.  Same operations in the same order.
+template <int PREC>
+__global__ void mixed_block_end_kernel(float4 *__restrict__ xs, MixedRing R, void *p_out,
+                                       const float4 *__restrict__ rs, int64_t vh, int block, const SolverScalars *S) {
+  pdl_enter();
+  const int code = S->x_code;
+  const int n = (code >> 4) == block ? (code & 15) : 0;
+  if (n == 0) return;  // halted before this block; uniform
+  const bool on = !S->halt;
+  const float b = S->beta_f;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= vh) return;
+  cf xv[4][3], pv[4][3];
+  load_f32(xs, vh, i, xv);
+#pragma unroll 2
+  for (int j = 0; j < n; ++j) {
+    const float a = S->alpha_h[j];
+    PT<PREC>::load_spinor(R.p[j], vh, i, pv);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      cf &x = xv[k / 3][k % 3];
+      x.re = fmaf(a, pv[k / 3][k % 3].re, x.re);
+      x.im = fmaf(a, pv[k / 3][k % 3].im, x.im);
+    }
+  }
+  store_f32(xs, vh, i, xv);
+  if (!on) return;
+  load_f32(rs, vh, i, xv);  // the last step's p is in pv: a block that has not halted has all its steps
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    cf &q = pv[k / 3][k % 3];
+    q.re = fmaf(b, q.re, xv[k / 3][k % 3].re);
+    q.im = fmaf(b, q.im, xv[k / 3][k % 3].im);
+  }
+  PT<PREC>::store_spinor(p_out, vh, i, pv);
 }
 
 template <int PREC>
@@ -110,13 +150,23 @@ __global__ void mixed_after_update_kernel(const double *partials, int n, SolverS
 
 static unsigned site_blocks(int64_t vh) { return (unsigned)((vh + kBlasThreads - 1) / kBlasThreads); }
 
-cudaError_t launch_mixed_xpay(int hop_prec, void *p, const float4 *rs, int64_t vh,
+cudaError_t launch_mixed_xpay(int hop_prec, void *p_out, const void *p, const float4 *rs, int64_t vh,
                               const SolverScalars *S, cudaStream_t s) {
   note_launch();
   if (hop_prec == PREC_F16N)
-    return launch_pdl(mixed_xpay_kernel<PREC_F16N>, site_blocks(vh), kBlasThreads, 0, s, p, rs, vh, S);
+    return launch_pdl(mixed_xpay_kernel<PREC_F16N>, site_blocks(vh), kBlasThreads, 0, s, p_out, p, rs, vh, S);
   else
-    return launch_pdl(mixed_xpay_kernel<PREC_F32>, site_blocks(vh), kBlasThreads, 0, s, p, rs, vh, S);
+    return launch_pdl(mixed_xpay_kernel<PREC_F32>, site_blocks(vh), kBlasThreads, 0, s, p_out, p, rs, vh, S);
+}
+
+cudaError_t launch_mixed_block_end(int hop_prec, float4 *xs, const MixedRing &R, void *p_out,
+                                   const float4 *rs, int64_t vh, int block, const SolverScalars *S, cudaStream_t s) {
+  note_launch();
+  if (hop_prec == PREC_F16N)
+    return launch_pdl(mixed_block_end_kernel<PREC_F16N>, site_blocks(vh), kBlasThreads, 0, s, xs, R, p_out, rs,
+                      vh, block, S);
+  return launch_pdl(mixed_block_end_kernel<PREC_F32>, site_blocks(vh), kBlasThreads, 0, s, xs, R, p_out, rs, vh,
+                    block, S);
 }
 
 cudaError_t launch_mixed_copy(int hop_prec, void *p, const float4 *rs, int64_t vh, cudaStream_t s) {

@@ -19,8 +19,10 @@ __device__ __forceinline__ float2 split_double(double v) {
   return make_float2(h, __double2float_rn(v - (double)h));
 }
 
-// alpha = rr / pAp; a non-positive or non-finite pAp ends the solve (breakdown)
-__device__ __forceinline__ void cg_alpha_step(double pAp, SolverScalars *S) {
+// alpha = rr / pAp; a non-positive or non-finite pAp ends the solve (breakdown).
+// x_code != 0: step (x_code & 15) - 1 of block x_code >> 4 of the inner
+// iterations; its alpha is recorded for the block's update of x_s.
+__device__ __forceinline__ void cg_alpha_step(double pAp, SolverScalars *S, int x_code) {
   S->pAp = pAp;
   if (!(pAp > 0.0) || !isfinite(pAp)) {
     S->done = 2;
@@ -33,6 +35,10 @@ __device__ __forceinline__ void cg_alpha_step(double pAp, SolverScalars *S) {
   S->malpha_dw = split_double(-a);
   S->alpha_f = (float)a;
   S->malpha_f = (float)-a;
+  if (x_code) {
+    S->alpha_h[(x_code & 15) - 1] = (float)a;
+    S->x_code = x_code;
+  }
 }
 
 // beta = rr_new / rr, the stopping test on rr_new and the iteration cap
@@ -122,8 +128,7 @@ __device__ __forceinline__ void hop_finish_scalars(const HopParams &P) {
   if (threadIdx.x == 0) {
     SolverScalars *S = P.fin_S;
     S->fin_count = 0;
-    if (P.fin == FIN_ALPHA) cg_alpha_step(v, S);
-    else if (P.fin == FIN_BETA) cg_beta_step(v, S);
+    if (P.fin == FIN_ALPHA) cg_alpha_step(v, S, P.x_code);
     else mixed_beta_step(v, S);
   }
 }

@@ -129,13 +129,11 @@ __global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
 
 // Low-precision form for the inner CG: Ap = a w + b H^dag t in FP32 registers
 // (never rounded to the storage precision), then the FP32 update of the
-// inner solution xs and residual rs with alpha_f, as the unfused update
-// kernel does, and ||rs||^2 per hop block.  Cut for five blocks per SM (six
+// inner residual rs with alpha_f and ||rs||^2 per hop block.  Cut for five blocks per SM (six
 // cost the FP16 solve 1.5% at 24^3x48).
 template <int PREC>
 __global__ void __launch_bounds__(kHopThreads, 5)
-    hop_lp_cg_kernel(const HopParams P, const void *__restrict__ p, float4 *__restrict__ xs,
-                     float4 *__restrict__ rs, const SolverScalars *__restrict__ S) {
+    hop_lp_cg_kernel(const HopParams P, float4 *__restrict__ rs, const SolverScalars *__restrict__ S) {
   typedef PT<PREC> T;
   extern __shared__ float4 lsm[];
   pdl_enter();
@@ -147,23 +145,17 @@ __global__ void __launch_bounds__(kHopThreads, 5)
     lp_hop_site<PREC, true, false>(lsm, P.in, reinterpret_cast<const float4 *>(P.gauge), P.g,
                                    P.out_parity, idx, acc);
     const float a = (float)P.a, b = (float)P.b, al = S->alpha_f;
-    cf w[4][3], pv[4][3], xv[4][3], rv[4][3];
+    cf w[4][3], rv[4][3];
     T::load_spinor(P.x, P.g.vh, idx, w);
-    T::load_spinor(p, P.g.vh, idx, pv);
-    PT<PREC_F32>::load_spinor(xs, P.g.vh, idx, xv);
     PT<PREC_F32>::load_spinor(rs, P.g.vh, idx, rv);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       const cf q = T::axpby(a, w[k / 3][k % 3], b, acc[k / 3][k % 3]);
-      cf &x = xv[k / 3][k % 3], &r = rv[k / 3][k % 3];
-      const cf pp = pv[k / 3][k % 3];
-      x.re = fmaf(al, pp.re, x.re);
-      x.im = fmaf(al, pp.im, x.im);
+      cf &r = rv[k / 3][k % 3];
       r.re = fmaf(-al, q.re, r.re);
       r.im = fmaf(-al, q.im, r.im);
       n2 = fmaf(r.re, r.re, fmaf(r.im, r.im, n2));
     }
-    PT<PREC_F32>::store_spinor(xs, P.g.vh, idx, xv);
     PT<PREC_F32>::store_spinor(rs, P.g.vh, idx, rv);
   }
   const double s = block_sum_f(n2);
@@ -172,21 +164,18 @@ __global__ void __launch_bounds__(kHopThreads, 5)
 }
 
 template <int PREC>
-cudaError_t launch_lp_cg_t(const HopParams &P, const void *p, float4 *xs, float4 *rs,
-                           const SolverScalars *S, cudaStream_t s) {
-  return launch_pdl(hop_lp_cg_kernel<PREC>, hop_blocks(P.g.vh), kHopThreads, lp_stage_smem<PREC>(), s, P, p,
-                    xs, rs, S);
+cudaError_t launch_lp_cg_t(const HopParams &P, float4 *rs, const SolverScalars *S, cudaStream_t s) {
+  return launch_pdl(hop_lp_cg_kernel<PREC>, hop_blocks(P.g.vh), kHopThreads, lp_stage_smem<PREC>(), s, P, rs, S);
 }
 
 }  // namespace
 
-cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, const void *p, float4 *xs, float4 *rs,
-                             const SolverScalars *S, cudaStream_t s) {
+cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, float4 *rs, const SolverScalars *S, cudaStream_t s) {
   note_launch();
   if (P.fin && (!P.fin_S || hop_blocks(P.g.vh) > (unsigned)JQCD_FIN_MAX_BLOCKS)) return cudaErrorInvalidValue;
   switch (prec) {
-    case PREC_F32: return launch_lp_cg_t<PREC_F32>(P, p, xs, rs, S, s);
-    case PREC_F16N: return launch_lp_cg_t<PREC_F16N>(P, p, xs, rs, S, s);
+    case PREC_F32: return launch_lp_cg_t<PREC_F32>(P, rs, S, s);
+    case PREC_F16N: return launch_lp_cg_t<PREC_F16N>(P, rs, S, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -16,7 +16,9 @@ inline unsigned hop_blocks(int64_t vh) { return (unsigned)((vh + kHopThreads - 1
 
 struct SolverScalars;
 // Scalar step the last block of a hop launch with norm takes (cg_steps.cuh)
-enum { FIN_NONE = 0, FIN_ALPHA = 1, FIN_BETA = 2, FIN_MIXED_BETA = 3 };
+enum { FIN_NONE = 0, FIN_ALPHA = 1, FIN_MIXED_BETA = 2 };
+// Inner iterations of the mixed CG between two updates of x_s
+constexpr int kMixedBlock = 8;
 // Grids of at most this many blocks take the scalar steps in their last block
 // instead of a separate single-block launch.
 #ifndef JQCD_FIN_MAX_BLOCKS
@@ -36,6 +38,7 @@ struct HopParams {
   const int *guard;   // when non-null and *guard != 0 the launch does nothing
   SolverScalars *fin_S;  // with fin != FIN_NONE (and norm): the scalars the last block updates
   int fin;
+  int x_code;            // FIN_ALPHA: as cg_alpha_step
 };
 
 // out_p = a x_p + b H_{p,1-p} in (dag: adjoint hop); partials get per-block
@@ -101,7 +104,8 @@ struct SolverScalars {
   int halt;         // loop kernels return at once while nonzero (done or need_update)
   int reliable_updates;
   int fin_count;    // blocks of the current hop launch that have written their partial
-  int pad1;
+  int x_code;       // inner CG: 16 * block of iterations + steps whose x_s += alpha p is due
+  float alpha_h[kMixedBlock];  // their alphas
 };
 
 // sum of partials[0..n) in a fixed order -> *out
@@ -140,9 +144,17 @@ cudaError_t launch_dw_to_f64(double2 *dst, const float4 *src, int64_t n, cudaStr
 cudaError_t launch_f64_to_dw(float4 *dst, const double2 *src, int64_t n, cudaStream_t s);
 
 // ---- mixed precision (inner CG in FP32 or FP16+norm, even parity) ----------
-// p = r_s + beta p in the hop precision (guarded)
-cudaError_t launch_mixed_xpay(int hop_prec, void *p, const float4 *rs, int64_t vh,
+// p_out = r_s + beta p in the hop precision (guarded; p_out may be p)
+cudaError_t launch_mixed_xpay(int hop_prec, void *p_out, const void *p, const float4 *rs, int64_t vh,
                               const SolverScalars *S, cudaStream_t s);
+// The directions of a block of inner iterations.
+struct MixedRing {
+  const void *p[kMixedBlock];
+};
+// The end of block `block` of iterations: x_s += alpha_j p_j for its steps,
+// and p_out = r_s + beta p of the last step unless the loop has halted.
+cudaError_t launch_mixed_block_end(int hop_prec, float4 *xs, const MixedRing &R, void *p_out,
+                                   const float4 *rs, int64_t vh, int block, const SolverScalars *S, cudaStream_t s);
 // p = r_s converted to the hop precision
 cudaError_t launch_mixed_copy(int hop_prec, void *p, const float4 *rs, int64_t vh, cudaStream_t s);
 // r_s = FP32(r) for a double-word r of vh sites
@@ -158,8 +170,9 @@ cudaError_t launch_mixed_beta(const double *partials, int n, SolverScalars *S, c
 cudaError_t launch_mixed_after_update(const double *partials, int n, SolverScalars *S,
                                       cudaStream_t s);
 
-// CG scalar steps (single block): alpha = rr / sum(partials)
-cudaError_t launch_cg_alpha(const double *partials, int n, SolverScalars *S, cudaStream_t s);
+// CG scalar steps (single block): alpha = rr / sum(partials); x_code as in
+// cg_alpha_step (0: not an inner iteration)
+cudaError_t launch_cg_alpha(const double *partials, int n, SolverScalars *S, cudaStream_t s, int x_code = 0);
 // rr_new = sum(partials); iters++; done when rr_new <= stop_rr; beta = rr_new/rr
 cudaError_t launch_cg_beta(const double *partials, int n, SolverScalars *S, cudaStream_t s);
 // S->rr = sum(partials) and reset the loop state (start or restart of CG)

@@ -291,27 +291,6 @@ cudaError_t GaugeEntry::ensure_multishift(int nshift) {
   return e;
 }
 
-// Residuals of a block of iterations beside vr: as many as up to kMsBlock - 1
-// that each take no more than a sixteenth of the free memory (blocks are
-// shorter with fewer; GaugeEntry::alloc gives them back when it runs out).
-void GaugeEntry::ensure_ms_ring() {
-  const size_t half = spinor_parity_bytes(PREC_DW, g.vh);
-  while ((int)ms_r.size() < kMsBlock - 1) {
-    size_t free_b = 0, total = 0;
-    void *p = nullptr;
-    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess || half > free_b / 16 || cudaMalloc(&p, half) != cudaSuccess) {
-      cudaGetLastError();
-      return;
-    }
-    ms_r.push_back((float4 *)p);
-  }
-}
-
-void GaugeEntry::drop_ms_ring() {
-  for (float4 *p : ms_r) cudaFree(p);
-  ms_r.clear();
-}
-
 jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshift, const double *shifts,
                              float4 *const *x_even, cudaStream_t s, jqcd_solve_info *infos,
                              std::string *msg) {
@@ -337,7 +316,8 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
     return JQCD_EINVAL;
   }
   CKM(G.ensure_multishift(nshift));
-  G.ensure_ms_ring();
+  // (after the caller's own allocations)
+  G.grow_ring(G.ms_r, spinor_parity_bytes(PREC_DW, G.g.vh), kMsBlock - 1);
   const int64_t vh = G.g.vh;
   const int64_t n = 12 * vh;  // complex double-word numbers of one parity
   const int nblas = (int)blas_blocks(n);
@@ -348,7 +328,7 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
   float4 *ring[kMsBlock];
   MsResiduals R;
   memset(&R, 0, sizeof R);
-  for (int j = 0; j < nring; ++j) R.r[j] = ring[j] = j + 1 < nring ? G.ms_r[j] : G.vec_even(G.vr);
+  for (int j = 0; j < nring; ++j) R.r[j] = ring[j] = j + 1 < nring ? (float4 *)G.ms_r[j] : G.vec_even(G.vr);
   const float4 *r_last = ring[nring - 1];  // the newest residual
   MsSteps *B = G.ms_B;
   MsVectors V;

@@ -30,7 +30,7 @@ constexpr int kMaxRestarts = 8;
 
 GaugeEntry::~GaugeEntry() {
   for (void *p : device_allocs) cudaFree(p);
-  drop_ms_ring();
+  drop_rings();
   if (S_host) cudaFreeHost(S_host);
   if (ms_S_host) cudaFreeHost(ms_S_host);
   if (ev0) cudaEventDestroy(ev0);
@@ -43,13 +43,36 @@ GaugeEntry::~GaugeEntry() {
 cudaError_t GaugeEntry::alloc(void **p, size_t bytes) {
   *p = nullptr;
   cudaError_t e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
-  if (e == cudaErrorMemoryAllocation && !ms_r.empty()) {
+  if (e == cudaErrorMemoryAllocation && drop_rings()) {
     cudaGetLastError();
-    drop_ms_ring();  // cudaFree waits for the device: nothing still reads them
     e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
   }
   if (e == cudaSuccess) device_allocs.push_back(*p);
   return e;
+}
+
+// Up to `most` vectors, each of no more than a sixteenth of the free memory.
+void GaugeEntry::grow_ring(std::vector<void *> &ring, size_t bytes, int most) {
+  while ((int)ring.size() < most) {
+    size_t free_b = 0, total = 0;
+    void *p = nullptr;
+    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess || bytes > free_b / 16 || cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    ring.push_back(p);
+  }
+}
+
+// (cudaFree waits for the device: nothing still reads them)
+bool GaugeEntry::drop_rings() {
+  bool any = false;
+  for (std::vector<void *> *r : {&ms_r, &mring[0], &mring[1]}) {
+    for (void *p : *r) cudaFree(p);
+    any = any || !r->empty();
+    r->clear();
+  }
+  return any;
 }
 
 cudaError_t GaugeEntry::ensure_canon() {
@@ -239,11 +262,11 @@ static bool fuse_scalar_steps(int nb) { return nb <= JQCD_FIN_MAX_BLOCKS; }
 // single-block step runs beside it; s waits for it before the last hop
 // (measured on GB300: double-word solve 33.62 -> 33.53 ms at 24^3x48, 4.48 ->
 // 4.39 ms at 16^4; mixed FP16 13.90 -> 13.81 ms).
-static cudaError_t alpha_fork(GaugeEntry &G, int nb, SolverScalars *S, cudaStream_t s) {
-  if (!G.side) return launch_cg_alpha(G.partials, nb, S, s);
+static cudaError_t alpha_fork(GaugeEntry &G, int nb, SolverScalars *S, cudaStream_t s, int x_code = 0) {
+  if (!G.side) return launch_cg_alpha(G.partials, nb, S, s, x_code);
   cudaError_t e = cudaEventRecord(G.ev_fork, s);
   if (!e) e = cudaStreamWaitEvent(G.side, G.ev_fork, 0);
-  if (!e) e = launch_cg_alpha(G.partials, nb, S, G.side);
+  if (!e) e = launch_cg_alpha(G.partials, nb, S, G.side, x_code);
   if (!e) e = cudaEventRecord(G.ev_join, G.side);
   return e;
 }
@@ -282,16 +305,27 @@ cudaError_t dw_eo_cg_iteration(GaugeEntry &G, double kappa, SolverScalars *S, cu
   return launch_dw_xpay(G.vp, G.vr, 12 * G.g.vh, S, s);
 }
 
-// One iteration of the inner CG of the mixed solver in hop precision hp on
-// the vectors p, t, w of that precision (FP32 xs and rs): the same order as
-// the double-word iteration, the update fused into the last hop.
-cudaError_t lp_eo_cg_iteration(GaugeEntry &G, int hp, int mk, double kappa, SolverScalars *S,
-                               cudaStream_t s) {
+// The directions of a block of inner iterations: step j reads p[j] and writes
+// the next direction to p[j + 1]; the pass that ends the block brings x_s up to
+// date (mixed_block_end_kernel) and writes p[0] of the next.
+struct InnerBlock {
+  void *p[kMixedBlock];
+  int m;          // directions there is room for: steps of a block
+  int id = 1;     // number of the block (27 bits)
+};
+
+// Step `slot` of a block of the inner CG of the mixed solver in hop precision
+// hp on the vectors p, t, w of that precision (FP32 xs and rs): the same order
+// as the double-word iteration, the residual update fused into the last hop.
+// end: this step ends its block.
+cudaError_t lp_eo_cg_iteration(GaugeEntry &G, int hp, int mk, double kappa, SolverScalars *S, InnerBlock &B, int slot,
+                               bool end, cudaStream_t s) {
   const double k2 = -kappa * kappa;
   const int nb = (int)hop_blocks(G.g.vh);
   const bool fuse = fuse_scalar_steps(nb);
   const int *guard = &S->halt;
-  void *p = G.mp[mk], *t = G.mt[mk], *w = G.mw[mk];
+  const int x_code = 16 * B.id + slot + 1;
+  void *p = B.p[slot], *t = G.mt[mk], *w = G.mw[mk];
   HopParams P = G.hop_params(hp, 1, p, nullptr, t, 0.0, 1.0, nullptr);
   P.guard = guard;
   cudaError_t e = launch_hop(hp, P, false, false, false, s);  // t = H_oe p
@@ -301,10 +335,11 @@ cudaError_t lp_eo_cg_iteration(GaugeEntry &G, int hp, int mk, double kappa, Solv
   if (fuse) {
     P.fin = FIN_ALPHA;
     P.fin_S = S;
+    P.x_code = x_code;
   }
   e = launch_hop(hp, P, false, true, true, s);  // w = p - k^2 H_eo t, ||w||^2
   if (e) return e;
-  if (!fuse && (e = alpha_fork(G, nb, S, s))) return e;
+  if (!fuse && (e = alpha_fork(G, nb, S, s, x_code))) return e;
   P = G.hop_params(hp, 1, w, nullptr, t, 0.0, 1.0, nullptr);
   P.guard = guard;
   e = launch_hop(hp, P, true, false, false, s);  // t = H^dag_oe w
@@ -316,10 +351,15 @@ cudaError_t lp_eo_cg_iteration(GaugeEntry &G, int hp, int mk, double kappa, Solv
     P.fin = FIN_MIXED_BETA;
     P.fin_S = S;
   }
-  e = launch_hop_lp_cg(hp, P, p, (float4 *)G.mx, (float4 *)G.mr, S, s);
+  e = launch_hop_lp_cg(hp, P, (float4 *)G.mr, S, s);
   if (e) return e;
   if (!fuse && (e = launch_mixed_beta(G.partials, nb, S, s))) return e;
-  return launch_mixed_xpay(hp, p, (const float4 *)G.mr, G.g.vh, S, s);
+  if (!end) return launch_mixed_xpay(hp, B.p[slot + 1], p, (const float4 *)G.mr, G.g.vh, S, s);
+  MixedRing R;
+  for (int j = 0; j < kMixedBlock; ++j) R.p[j] = j < B.m ? B.p[j] : nullptr;
+  e = launch_mixed_block_end(hp, (float4 *)G.mx, R, B.p[0], (const float4 *)G.mr, G.g.vh, B.id, S, s);
+  B.id = B.id < (1 << 26) ? B.id + 1 : 1;
+  return e;
 }
 
 // ---- native FP64 system (JQCD_CG_F64) -------------------------------------
@@ -390,7 +430,13 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
       return e_ == cudaErrorMemoryAllocation ? JQCD_ENOMEM : JQCD_ECUDA; \
     }                                                          \
   } while (0)
-  if (mixed) CKS(G.ensure_mixed(hp));
+  InnerBlock IB;
+  if (mixed) {
+    CKS(G.ensure_mixed(hp));
+    G.grow_ring(G.mring[mk], spinor_parity_bytes(hp, vh), kMixedBlock - 1);
+    IB.m = 1 + (int)G.mring[mk].size();
+    for (int j = 0; j < IB.m; ++j) IB.p[j] = j ? G.mring[mk][j - 1] : G.mp[mk];
+  }
 
   CKS(cudaEventRecord(G.ev0, s));
   CKS(cudaMemsetAsync(S, 0, sizeof(SolverScalars), s));
@@ -431,7 +477,7 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
     if (!mixed) return launch_dw_copy(G.vp, G.vr, A.n, s);
     cudaError_t e = launch_dw_to_f32((float4 *)G.mr, G.vr, vh, s);
     if (!e) e = cudaMemsetAsync(G.mx, 0, spinor_parity_bytes(PREC_F32, vh), s);
-    if (!e) e = launch_mixed_copy(hp, G.mp[mk], (const float4 *)G.mr, vh, s);
+    if (!e) e = launch_mixed_copy(hp, IB.p[0], (const float4 *)G.mr, vh, s);
     return e;
   };
   CKS(start_direction());
@@ -451,7 +497,8 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
           CKS(launch_cg_beta(G.partials, nblas, S, s));
           CKS(launch_dw_xpay(G.vp, G.vr, A.n, S, s));
         } else {
-          CKS(lp_eo_cg_iteration(G, hp, mk, P.kappa, S, s));
+          const int slot = k % IB.m;
+          CKS(lp_eo_cg_iteration(G, hp, mk, P.kappa, S, IB, slot, slot + 1 == IB.m || k + 1 == kCheckEvery, s));
         }
       }
       CKS(cudaMemcpyAsync(G.S_host, S, sizeof(SolverScalars), cudaMemcpyDeviceToHost, s));
@@ -463,7 +510,9 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
         CKS(launch_dw_xmy_norm(G.vr, G.vrhs, G.vAp, A.n, G.partials, s));
         CKS(launch_mixed_after_update(G.partials, nblas, S, s));
         CKS(launch_dw_to_f32((float4 *)G.mr, G.vr, vh, s));
-        CKS(launch_mixed_xpay(hp, G.mp[mk], (const float4 *)G.mr, vh, S, s));
+        // p = r + beta p from the direction of the iteration that halted
+        const int steps = G.S_host->x_code & 15;
+        CKS(launch_mixed_xpay(hp, IB.p[0], IB.p[steps - 1], (const float4 *)G.mr, vh, S, s));
         CKS(cudaMemcpyAsync(G.S_host, S, sizeof(SolverScalars), cudaMemcpyDeviceToHost, s));
         CKS(cudaStreamSynchronize(s));
       }

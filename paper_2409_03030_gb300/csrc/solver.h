@@ -26,9 +26,11 @@ struct GaugeEntry {
   float4 *vb = nullptr, *vsol = nullptr, *vr = nullptr, *vp = nullptr, *vAp = nullptr,
          *vw = nullptr, *vt = nullptr, *vrhs = nullptr;
   // mixed-precision inner vectors (even parity): x, r in FP32; p, w in the
-  // hop precision; t odd in the hop precision
+  // hop precision; t odd in the hop precision; mring: directions of a block of
+  // iterations beside mp
   void *mx = nullptr, *mr = nullptr, *mp[2] = {nullptr, nullptr}, *mw[2] = {nullptr, nullptr},
        *mt[2] = {nullptr, nullptr};
+  std::vector<void *> mring[2];
   // native FP64 solver vectors (whole lattice)
   double2 *fb = nullptr, *fsol = nullptr, *fr = nullptr, *fp = nullptr, *fAp = nullptr,
           *fw = nullptr, *ft = nullptr, *frhs = nullptr;
@@ -38,7 +40,7 @@ struct GaugeEntry {
   double *lcanon = nullptr;
   // multi-shift CG workspace: per-shift search directions and scalars
   std::vector<float4 *> ms_p, ms_x;  // ms_x: solutions of the host-buffer entry
-  std::vector<float4 *> ms_r;        // residuals of a block of iterations, beside vr
+  std::vector<void *> ms_r;          // residuals of a block of iterations, beside vr
   MsScalars *ms_S = nullptr;
   MsSteps *ms_B = nullptr;
   MsScalars *ms_S_host = nullptr;  // pinned mirror
@@ -80,8 +82,10 @@ struct GaugeEntry {
   cudaError_t ensure_f64();
   cudaError_t ensure_force();
   cudaError_t ensure_multishift(int nshift);
-  void ensure_ms_ring();
-  void drop_ms_ring();
+  // vectors that only make blocks of iterations longer: allocated while there
+  // is room for them, given back when another allocation runs out
+  void grow_ring(std::vector<void *> &ring, size_t bytes, int most);
+  bool drop_rings();
   cudaError_t ensure_staggered();
   cudaError_t ensure_hmc();
   // fermion-solve history of a trajectory: previous X, Y and two start vectors
@@ -117,10 +121,9 @@ cudaError_t launch_hop_dw_r(const HopParams &P, const float4 *r_in, float4 *r, c
                             cudaStream_t s);
 
 // The same for the inner CG of the mixed solver in hop precision prec (FP32 or
-// FP16 with norm): p, t and w in that precision, xs and rs FP32, alpha =
+// FP16 with norm), without x: t and w in that precision, rs FP32, alpha =
 // S->alpha_f.
-cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, const void *p, float4 *xs, float4 *rs,
-                             const SolverScalars *S, cudaStream_t s);
+cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, float4 *rs, const SolverScalars *S, cudaStream_t s);
 
 // Run the solve of D x = b for the double-word b in G.vb; the solution is
 // left in G.vsol (whole lattice, double-word).  Mode JQCD_CG_F64 widens b to
