@@ -202,59 +202,54 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS) hop_dwp_ker
   }
 }
 
-// Small lattices: two threads per output site (dwp_pair_combine), so the
-// grid holds twice as many warps when one thread per site cannot fill the
-// GPU.  Blocks of kDwp2Threads threads cover kDwp2Threads / 2 sites.
+// Small lattices: eight threads per output site (dwp8_hop).  A hop there is a
+// latency chain, the loads' round trip and the arithmetic of as many hops as a
+// thread runs, on too few warps to hide it: with one hop per thread, 8^4 (two
+// threads: 5.3 us back to back) takes 2.7 us, 12^4 (8.3 us) 6.0 us.
 template <bool DAG, bool AXPY, bool NORM>
-__global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS) hop_dwp2_kernel(const HopParams P) {
-  extern __shared__ float4 dsm[];
+__global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS) hop_dwp8_kernel(const HopParams P) {
+  __shared__ ulonglong2 sm[6][kDwp8Threads];
   pdl_wait();
   if (P.guard && *P.guard) return;  // uniform across the grid
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t idx = gid >> 1;
-  const int q = (int)(gid & 1);
-  const bool active = idx < P.g.vh;  // the same for both threads of a site
-  p2 acc[4][3];
-  if (active) {
-    dwp_hop_dirs<DAG, kDwp2Threads, 4, 2>(dsm, reinterpret_cast<const float4 *>(P.in),
-                                                reinterpret_cast<const float4 *>(P.gauge), P.g, P.out_parity,
-                                                (unsigned)idx, q, acc);
-  } else {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[a][c] = p2{0ull, 0ull};
-  }
-  pdl_trigger();  // the split grid is less than one wave
-  p2 o[6];
-  dwp_pair_combine(acc, q, o);  // every lane of the warp takes part
+  const int64_t base = (int64_t)blockIdx.x * kDwp8Sites;
+  const int64_t hop_idx = base + (threadIdx.x & 15);
+  if (hop_idx < P.g.vh)
+    dwp8_hop<DAG>(sm, reinterpret_cast<const float4 *>(P.in), reinterpret_cast<const float4 *>(P.gauge), P.g,
+                  P.out_parity, (unsigned)hop_idx);
+  pdl_trigger();
+  __syncthreads();
   dwacc nrm{0.f, 0.f};
-  if (active)
-    nrm = dwp_store_chunks<AXPY, NORM, 6>(o, 6 * q, reinterpret_cast<float4 *>(P.out),
-                                          reinterpret_cast<const float4 *>(P.x), P.g.vh, idx,
-                                          P.a_split, P.b_split);
+  const int j = threadIdx.x & 15, spin = threadIdx.x >> 4;
+  if (spin < 4 && base + j < P.g.vh) {
+    p2 v[3];
+    dwp8_sum<DAG>(sm, j, spin, v);
+    nrm = dwp_store_chunks<AXPY, NORM, 3>(v, 3 * spin, reinterpret_cast<float4 *>(P.out),
+                                          reinterpret_cast<const float4 *>(P.x), P.g.vh, base + j, P.a_split,
+                                          P.b_split);
+  }
   if (NORM) {
     const double s = block_sum_dw(nrm);
     if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
   }
 }
 
-// Two threads per site pay off only while their grid fits in one wave of
-// resident warps (measured on GB300: 8^4 hop 9.6 -> 5.9 us; at 16^4, where
-// the split grid needs 1.12 waves, 19.1 -> 18.6 us and the solve slower;
-// 16^3x32 at 2.25 waves 24.8 -> 30.4 us).  Twelve warps per SM is the most
-// the split kernel's 164-168 registers allow: a thirteenth puts a fourth
-// warp on one SM sub-partition, whose register file then caps every thread
-// at 128 registers (the kernel spilled 402 bytes and ran 25-40% slower).
-bool dw_hop_split(int64_t vh) {
+// Eight threads per site up to SMs x JQCD_DWP8_BLOCKS blocks of 16 sites
+// (29184 sites per parity).  Measured on GB300, Mhat^dag Mhat p with its norm
+// and the solve, against the two threads per site that ran there before: 8^4
+// 28.9 -> 22.5 us and 1.90 -> 1.58 ms, 12^4 40.9 -> 31.3 us and 2.95 -> 2.55
+// ms, 16^3x12 58.7 -> 52.2 us and 4.18 -> 3.94 ms, 16^3x14 60.1 -> 58.2 us and
+// 4.47 -> 4.41 ms.  One thread per site takes 55.2 us and 4.08 ms at 16^3x12,
+// 55.6 us and 4.32 ms at 16^3x14 (but its sum of eight hops in a row has a 5%
+// larger rounding error), and wins at 16^4 (56.6 against 67.6 us).
+bool dw_hop_split8(int64_t vh) {
   static const int64_t max_vh = [] {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
       return (int64_t)0;
-    return (int64_t)sms * JQCD_DWP2_MIN_BLOCKS * kDwp2Threads / 2;
+    return (int64_t)sms * JQCD_DWP8_BLOCKS * kDwp8Sites;
   }();
-  return vh <= max_vh && vh <= JQCD_DWP_SPLIT_MAX_VH;
+  return vh <= max_vh;
 }
 
 // A one-thread grid of at most SMs x JQCD_DWP_SMALL_BLOCKS blocks is launched
@@ -275,12 +270,12 @@ bool dw_hop_small(int64_t vh) {
       return (int64_t)0;
     return (int64_t)sms * JQCD_DWP_SMALL_BLOCKS * kDwp1Threads;
   }();
-  return !dw_hop_split(vh) && vh <= max_vh && vh <= JQCD_DWP_SMALL_MAX_VH;
+  return !dw_hop_split8(vh) && vh <= max_vh && vh <= JQCD_DWP_SMALL_MAX_VH;
 }
 
 unsigned dw_hop_blocks(int64_t vh) {
-  return dw_hop_split(vh) ? (unsigned)((2 * vh + kDwp2Threads - 1) / kDwp2Threads)
-                          : (unsigned)((vh + kDwp1Threads - 1) / kDwp1Threads);
+  if (dw_hop_split8(vh)) return (unsigned)((vh + kDwp8Sites - 1) / kDwp8Sites);
+  return (unsigned)((vh + kDwp1Threads - 1) / kDwp1Threads);
 }
 
 unsigned hop_norm_partials(int prec, int64_t vh) {
@@ -292,15 +287,14 @@ static cudaError_t launch_hop_dw_t(const HopParams &P, cudaStream_t s) {
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
   auto kern = hop_dwp_kernel<DAG, AXPY, NORM>;
-  auto kern2 = hop_dwp2_kernel<DAG, AXPY, NORM>;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwp2Smem);
+    const cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  if (dw_hop_split(P.g.vh)) return launch_pdl(kern2, dw_hop_blocks(P.g.vh), kDwp2Threads, kDwp2Smem, s, P);
+  if (dw_hop_split8(P.g.vh))
+    return launch_pdl(hop_dwp8_kernel<DAG, AXPY, NORM>, dw_hop_blocks(P.g.vh), kDwp8Threads, 0, s, P);
   return launch_pdl(kern, dw_hop_blocks(P.g.vh), kDwp1Threads, dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s,
                     P);
 }

@@ -92,37 +92,29 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
   if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
 }
 
-// The same with two threads per output site (small lattices, see
-// dwp_pair_combine): thread q updates components 6q .. 6q + 5.
+// The same with eight threads per output site (small lattices, dw_hop_split8).
 template <bool XUPD>
-__global__ void __launch_bounds__(kDwp2Threads, JQCD_DWP2_MIN_BLOCKS)
-    hop_dwp2_cg_kernel(const HopParams P, const float4 *__restrict__ p, float4 *__restrict__ xs,
+__global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS)
+    hop_dwp8_cg_kernel(const HopParams P, const float4 *__restrict__ p, float4 *__restrict__ xs,
                        const float4 *r_in, float4 *r, const float2 *__restrict__ alpha) {
-  extern __shared__ float4 dsm[];
+  __shared__ ulonglong2 sm[6][kDwp8Threads];
   pdl_wait();
   if (P.guard && *P.guard) return;  // uniform across the grid
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t idx = gid >> 1;
-  const int q = (int)(gid & 1);
-  const bool active = idx < P.g.vh;
-  p2 acc[4][3];
-  if (active) {
-    dwp_hop_dirs<true, kDwp2Threads, 4, 2>(dsm, reinterpret_cast<const float4 *>(P.in),
-                                                 reinterpret_cast<const float4 *>(P.gauge), P.g, P.out_parity,
-                                                 (unsigned)idx, q, acc);
-  } else {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc[a][c] = p2{0ull, 0ull};
-  }
-  pdl_trigger();  // the split grid is less than one wave
-  p2 o[6];
-  dwp_pair_combine(acc, q, o);
+  const int64_t base = (int64_t)blockIdx.x * kDwp8Sites;
+  const int64_t hop_idx = base + (threadIdx.x & 15);
+  if (hop_idx < P.g.vh)
+    dwp8_hop<true>(sm, reinterpret_cast<const float4 *>(P.in), reinterpret_cast<const float4 *>(P.gauge), P.g,
+                   P.out_parity, (unsigned)hop_idx);
+  pdl_trigger();
+  __syncthreads();
   dwacc nrm{0.f, 0.f};
-  if (active)
-    nrm = dwp_store_cg<XUPD, 6>(o, 6 * q, reinterpret_cast<const float4 *>(P.x), p, xs, r_in, r, P.g.vh, idx,
-                                P.a_split, P.b_split, *alpha);
+  const int j = threadIdx.x & 15, spin = threadIdx.x >> 4;
+  if (spin < 4 && base + j < P.g.vh) {
+    p2 v[3];
+    dwp8_sum<true>(sm, j, spin, v);
+    nrm = dwp_store_cg<XUPD, 3>(v, 3 * spin, reinterpret_cast<const float4 *>(P.x), p, xs, r_in, r, P.g.vh,
+                                base + j, P.a_split, P.b_split, *alpha);
+  }
   const double s = block_sum_dw(nrm);
   if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
 }
@@ -186,17 +178,13 @@ static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kDwpSmallSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(hop_dwp2_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kDwp2Smem);
+    const cudaError_t e = cudaFuncSetAttribute(
+        hop_dwp_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  if (dw_hop_split(P.g.vh))
-    return launch_pdl(hop_dwp2_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp2Threads, kDwp2Smem, s, P, p, x,
-                      r_in, r, alpha);
+  if (dw_hop_split8(P.g.vh))
+    return launch_pdl(hop_dwp8_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp8Threads, 0, s, P, p, x, r_in, r, alpha);
   return launch_pdl(hop_dwp_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp1Threads,
                     dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P, p, x, r_in, r, alpha);
 }

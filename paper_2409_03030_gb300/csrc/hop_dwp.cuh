@@ -28,11 +28,7 @@ constexpr size_t kDwpSmem = dwp_smem();
 
 // Launch shapes of the single-field kernels: threads per block and the
 // resident blocks per SM their register budget is cut for, one thread per
-// output site (DWP) and two (DWP2, small lattices).  One-warp blocks spread
-// a small lattice's split grid over more SMs (measured on GB300: 8^4 hop
-// 7.35 -> 5.87 us, 12^4 10.9 -> 8.85 us against 128-thread blocks).  The
-// one-thread kernel keeps 128: with one-warp blocks its plain hop ran 1%
-// faster at 24^3x48 but the solve 1.2% slower (four times the norm partials).
+// output site (DWP) and eight (DWP8, small lattices: dwp8_hop).
 #ifndef JQCD_DWP_THREADS
 #define JQCD_DWP_THREADS 128
 #endif
@@ -46,29 +42,26 @@ constexpr size_t kDwpSmem = dwp_smem();
 #ifndef JQCD_DWP_SMALL_BLOCKS
 #define JQCD_DWP_SMALL_BLOCKS 2
 #endif
-#ifndef JQCD_DWP2_THREADS
-#define JQCD_DWP2_THREADS 32
+#ifndef JQCD_DWP8_MIN_BLOCKS
+#define JQCD_DWP8_MIN_BLOCKS 4
 #endif
-#ifndef JQCD_DWP2_MIN_BLOCKS
-#define JQCD_DWP2_MIN_BLOCKS 12
+#ifndef JQCD_DWP8_BLOCKS
+#define JQCD_DWP8_BLOCKS 12
 #endif
 constexpr int kDwp1Threads = JQCD_DWP_THREADS;
 constexpr size_t kDwp1Smem = dwp_smem(kDwp1Threads);
 // 227 KB of shared memory per SM, 1 KB of it reserved per block
 constexpr size_t kDwpSmallSmem = (size_t)(227 / JQCD_DWP_SMALL_BLOCKS - 2) * 1024;
 static_assert(kDwpSmallSmem >= kDwp1Smem, "the limit only pads the stages");
-constexpr int kDwp2Threads = JQCD_DWP2_THREADS;
-constexpr size_t kDwp2Smem = dwp_smem(kDwp2Threads);
 
 // Issue the copies of a spinor (byte offset off) into its stage column st
 // (NT: threads per block, the stride of the chunk-major stage).  The chunk
 // planes in + k vh are uniform over the grid, so the per-thread part of every
-// address is the one 32-bit offset.  L1: through L1, where the neighbours of a
-// few resident warps find each other's spinors, or past it.
-template <int NT, bool L1>
+// address is the one 32-bit offset.
+template <int NT>
 __device__ __forceinline__ void stage_hop_p(float4 *st, const float4 *in, int64_t vh, unsigned off) {
 #pragma unroll
-  for (int k = 0; k < 12; ++k) cp_async16(st + k * NT, chunk_at(in + k * vh, off), L1);
+  for (int k = 0; k < 12; ++k) cp_async16(st + k * NT, chunk_at(in + k * vh, off), false);
 }
 
 // Issue the copies of the link of hop d (mu = d/2, backward when d is odd)
@@ -234,11 +227,10 @@ __device__ __forceinline__ void reconstruct_half_mu(int mu, const p2 (&r)[3], p2
   }
 }
 
-// acc = the sum over the ND hops d = d0, d0 + DSTEP, ... (hop d has mu = d/2
-// and is backward when d is odd) of H_{p,1-p} in at output site idx of parity
-// p (DAG: the adjoint hop), unnormalised double-word accumulators.  All eight
-// hops (d0 = 0, DSTEP = 1, ND = 8) give (H_{p,1-p} in)(idx).  dsm: this
-// block's dwp_smem(NT) bytes of shared memory; blockDim.x must be NT.
+// acc = (H_{p,1-p} in)(idx) at output site idx of parity p (DAG: the adjoint
+// hop), unnormalised double-word accumulators: all eight hops d = 2 mu +
+// backward in one thread.  dsm: this block's dwp_smem(NT) bytes of shared
+// memory; blockDim.x must be NT.
 //
 // Copies run one hop ahead: the link of the next hop is issued when hop d
 // starts (two link stages), the neighbour spinor of the next hop as soon as
@@ -246,63 +238,46 @@ __device__ __forceinline__ void reconstruct_half_mu(int mu, const p2 (&r)[3], p2
 // thread reads and overwrites only its own column, so no block barrier is
 // needed; the completed-group wait of each hop covers both of its copies.
 //
-// All eight hops in one thread (DSTEP 1): a runtime loop, whose body exists
-// once in the instruction stream; the neighbour offsets wait in shared
-// memory, one load per hop.  Computing each hop's neighbour and its 64-bit
-// chunk addresses in the loop instead took 49 of 748 instructions per hop and
-// warp, and the kernel is bound by issue and dependency latency at 12 warps
-// per SM.  With the spinor copies past L1 (cp.async.cg: three blocks' stages
-// leave L1 about 56 KB, less than the spinor bytes in flight, so allocating
-// there limited them): 97.9 -> 91.5 us at 24^3x48, 286.8 -> 265.1 us at
-// 32^3x64 (5.57 and 6.08 TB/s algorithmic, 82% and 90% of the measured copy
-// bandwidth).
-// Every other hop (DSTEP 2, two threads per site on small lattices): the four
-// hops unrolled with their offsets in registers; each SM's few warps are bound
-// by the latency of their own chain, and their directions are then constants
-// (12^4 solve 3.08 -> 2.99 ms); L1 is large beside their small stages and keeps
-// the spinors (past L1 the 14^4 solve takes 4.48 instead of 3.75 ms).
-template <bool DAG, int NT, int ND, int DSTEP>
-__device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, const float4 *gauge,
-                                             const Geom &g, int p, unsigned idx, int d0,
-                                             p2 (&acc)[4][3]) {
+// A runtime loop, whose body exists once in the instruction stream; the
+// neighbour offsets wait in shared memory, one load per hop.  Computing each
+// hop's neighbour and its 64-bit chunk addresses in the loop instead took 49
+// of 748 instructions per hop and warp, and the kernel is bound by issue and
+// dependency latency at 12 warps per SM.  The spinor copies go past L1: three
+// blocks' stages leave it about 56 KB, less than the spinor bytes in flight,
+// so allocating there limited them.  97.9 -> 91.2 us at 24^3x48, 286.8 ->
+// 265.1 us at 32^3x64 (5.59 and 6.08 TB/s algorithmic, 83% and 90% of the
+// measured copy bandwidth).
+template <bool DAG, int NT = kHopThreads>
+__device__ __forceinline__ void dwp_hop_site(float4 *dsm, const float4 *in, const float4 *gauge,
+                                             const Geom &g, int p, int64_t idx, p2 (&acc)[4][3]) {
   const int64_t vh = g.vh;
   const int tid = threadIdx.x;
   float4 *const spn = dsm + tid;                     // this thread's column of the spinor stage
   float4 *const lnk = spn + kDwpStageChunks * NT;    // and of the two link stages
   unsigned *const tab = reinterpret_cast<unsigned *>(dsm + (kDwpStageChunks + 2 * kDwpLinkChunks) * NT) + tid;
-  unsigned off[8];
   {
-    const HopSite site = hop_site(g, idx, p);
+    const HopSite site = hop_site(g, (unsigned)idx, p);
 #pragma unroll
-    for (int d = 0; d < 8; ++d) off[d] = hop_offset(g, site, d);
+    for (int d = 0; d < 8; ++d) tab[d * NT] = hop_offset(g, site, d);
   }
-  if (DSTEP == 1) {
-#pragma unroll
-    for (int d = 0; d < 8; ++d) tab[d * NT] = off[d];
-  }
-  auto offset = [&](int j) -> unsigned {  // of the j-th hop
-    if (DSTEP == 1) return tab[j * NT];
-    return d0 ? off[(2 * j + 1) & 7] : off[(2 * j) & 7];
-  };
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[a][c] = p2{0ull, 0ull};
-  const unsigned own = idx * 16u;
-  unsigned next = offset(0);
-  stage_hop_p<NT, DSTEP == 2>(spn, in, vh, next & ~1u);
-  stage_link_p<NT>(lnk, gauge, vh, p, d0, own, next & ~1u);
+  const unsigned own = 16u * (unsigned)idx;
+  unsigned next = tab[0];
+  stage_hop_p<NT>(spn, in, vh, next & ~1u);
+  stage_link_p<NT>(lnk, gauge, vh, p, 0, own, next & ~1u);
   cp_async_commit();
-#pragma unroll(DSTEP == 2 ? ND : 1)
-  for (int j = 0; j < ND; ++j) {
-    const int d = DSTEP == 1 ? j : d0 + j * DSTEP;
+#pragma unroll 1
+  for (int d = 0; d < 8; ++d) {
     const bool neg = next & 1u;
-    const int mu = DSTEP == 2 ? j : d >> 1;
+    const int mu = d >> 1;
     const bool bwd = (d & 1) != 0;
-    const bool more = j + 1 < ND;
+    const bool more = d < 7;
     if (more) {  // the other link stage was read during the previous hop
-      next = offset(j + 1);
-      stage_link_p<NT>(lnk + ((j + 1) & 1) * kDwpLinkChunks * NT, gauge, vh, p, d + DSTEP, own, next & ~1u);
+      next = tab[(d + 1) * NT];
+      stage_link_p<NT>(lnk + ((d + 1) & 1) * kDwpLinkChunks * NT, gauge, vh, p, d + 1, own, next & ~1u);
     }
     cp_async_commit();
     cp_async_wait1();  // this thread's spinor and link copies of hop d have landed
@@ -311,7 +286,7 @@ __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, cons
     for (int k = 0; k < 12; ++k) psi[k / 3][k % 3] = ld_p2(spn + k * NT);
     p2 W[3][3];
     {  // U_mu(x), or the transpose of U_mu(x - mu)
-      const float4 *ls = lnk + (j & 1) * kDwpLinkChunks * NT;
+      const float4 *ls = lnk + (d & 1) * kDwpLinkChunks * NT;
       const int sa = bwd ? NT : 3 * NT, sb = bwd ? 3 * NT : NT;
 #pragma unroll
       for (int k = 0; k < 9; ++k) W[k / 3][k % 3] = ld_p2(ls + (k / 3) * sa + (k % 3) * sb);
@@ -324,7 +299,7 @@ __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, cons
       case 2: project_p<2>(psi, h, S); break;
       default: project_p<3>(psi, h, S);
     }
-    if (more) stage_hop_p<NT, DSTEP == 2>(spn, in, vh, next & ~1u);  // the spinor stage has been read
+    if (more) stage_hop_p<NT>(spn, in, vh, next & ~1u);  // the spinor stage has been read
     cp_async_commit();
     if (neg) {
 #pragma unroll
@@ -350,27 +325,113 @@ __device__ __forceinline__ void dwp_hop_dirs(float4 *dsm, const float4 *in, cons
   }
 }
 
-// (H_{p,1-p} in)(idx): all eight hops in one thread.
-template <bool DAG, int NT = kHopThreads>
-__device__ __forceinline__ void dwp_hop_site(float4 *dsm, const float4 *in, const float4 *gauge,
-                                             const Geom &g, int p, int64_t idx, p2 (&acc)[4][3]) {
-  dwp_hop_dirs<DAG, NT, 8, 1>(dsm, in, gauge, g, p, (unsigned)idx, 0, acc);
+// Eight threads per output site (small lattices): a block of
+// kDwp8Threads threads covers kDwp8Sites sites, warp mu runs direction mu, its
+// lanes 0..15 the forward and 16..31 the backward hop of sites 0..15.  Each
+// thread loads its operands straight into registers (one round trip for all
+// of them), leaves its two-spin product in shared memory, and the first
+// 4 x kDwp8Sites threads sum one spin of one site each (dwp8_spin).  A hop's
+// latency chain is then one hop long.
+constexpr int kDwp8Sites = 16;
+constexpr int kDwp8Threads = 8 * kDwp8Sites;
+
+// This thread's r = W h into sm[3 s + c][thread] (see above); idx: its site.
+template <bool DAG>
+__device__ __forceinline__ void dwp8_hop(ulonglong2 (*sm)[kDwp8Threads], const float4 *in, const float4 *gauge,
+                                         const Geom &g, int p, unsigned idx) {
+  const int64_t vh = g.vh;
+  const int mu = threadIdx.x >> 5;
+  const bool bwd = (threadIdx.x & 16) != 0;
+  const HopSite site = hop_site(g, idx, p);
+  unsigned off;
+  switch (mu) {
+    case 0: off = bwd ? hop_offset(g, site, 1) : hop_offset(g, site, 0); break;
+    case 1: off = bwd ? hop_offset(g, site, 3) : hop_offset(g, site, 2); break;
+    case 2: off = bwd ? hop_offset(g, site, 5) : hop_offset(g, site, 4); break;
+    default: off = bwd ? hop_offset(g, site, 7) : hop_offset(g, site, 6);
+  }
+  const bool neg = off & 1u;
+  off &= ~1u;
+  p2 psi[4][3], W[3][3], h[2][3];
+  const float4 *L = gauge + (int64_t)(((bwd ? 1 - p : p) * 4 + mu) * 9) * vh;
+  const unsigned lo = bwd ? off : 16u * idx;
+  const int sa = bwd ? 1 : 3, sb = bwd ? 3 : 1;  // U_mu(x), or the transpose of U_mu(x - mu)
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(chunk_at(in + k * vh, off)));
+    psi[k / 3][k % 3] = p2{v.x, v.y};
+  }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const ulonglong2 v =
+        __ldg(reinterpret_cast<const ulonglong2 *>(chunk_at(L + ((k / 3) * sa + (k % 3) * sb) * vh, lo)));
+    W[k / 3][k % 3] = p2{v.x, v.y};
+  }
+  const float S = (bwd != DAG) ? 1.f : -1.f;
+  switch (mu) {
+    case 0: project_p<0>(psi, h, S); break;
+    case 1: project_p<1>(psi, h, S); break;
+    case 2: project_p<2>(psi, h, S); break;
+    default: project_p<3>(psi, h, S);
+  }
+  if (neg) {
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) h[a][c] = p2_neg(h[a][c]);
+  }
+  const f2 cj = bwd ? 0x8000000000000000ull : 0ull;  // conjugates the adjoint link
+#pragma unroll
+  for (int k = 0; k < 9; ++k) W[k / 3][k % 3] = p2{W[k / 3][k % 3].h ^ cj, W[k / 3][k % 3].l ^ cj};
+  const float wmax = link_max_hi(W) * 1.0000019f;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    p2 r[3];
+    matvec_half_p(W, wmax, h[s], r);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sm[3 * s + c][threadIdx.x] = make_ulonglong2(r[c].h, r[c].l);
+  }
 }
 
-// Two threads per output site (lanes 2i and 2i + 1 of a warp, q = lane & 1):
-// thread q runs the forward (q = 0) or backward (q = 1) hops of the four
-// directions, then the pair exchanges partial sums so that thread q holds
-// the whole result of spins 2q and 2q + 1, components 6q .. 6q + 5 in the
-// order of the spinor layout.  Every lane of the warp must call this.
-__device__ __forceinline__ void dwp_pair_combine(const p2 (&acc)[4][3], int q, p2 (&o)[6]) {
+// acc = spin SP of (H in) at site j of the block: the forward and the backward
+// hops' sums, added (shorter chains than all eight in a row, and on average a
+// smaller rounding error: 6.41e-14 against 6.76e-14 at 12^4).
+// The terms are those of reconstruct_half_p; the first of each sum is taken as
+// it is.
+template <bool DAG, int SP>
+__device__ __forceinline__ void dwp8_spin(const ulonglong2 (*sm)[kDwp8Threads], int j, p2 (&acc)[3]) {
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    const p2 up = acc[k / 3][k % 3], dn = acc[2 + k / 3][k % 3];
-    const p2 keep = q ? dn : up, send = q ? up : dn;
-    p2 recv;
-    recv.h = __shfl_xor_sync(0xffffffffu, send.h, 1);
-    recv.l = __shfl_xor_sync(0xffffffffu, send.l, 1);
-    o[k] = p2_add(keep, recv);
+  for (int c = 0; c < 3; ++c) {
+    p2 sum[2];
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {  // everything but the data is constant after unrolling
+      const int mu = d >> 1;
+      const int src = SP < 2 ? SP : (mu < 2 ? 3 - SP : SP - 2);
+      const ulonglong2 v = sm[3 * src + c][16 * d + j];
+      p2 r{v.x, v.y};
+      f2 sg = f2_make(1.f, 1.f);
+      if (SP >= 2) {
+        const float S = (((d & 1) != 0) != DAG) ? 1.f : -1.f;
+        if (!(mu & 1)) r = p2_swap(r);
+        if (mu == 0 || (mu == 2 && SP == 2)) sg = f2_make(S, -S);
+        if (mu == 2 && SP == 3) sg = f2_make(-S, S);
+        if (mu == 3 || (mu == 1 && SP == 2)) sg = f2_make(S, S);
+        if (mu == 1 && SP == 3) sg = f2_make(-S, -S);
+      }
+      p2 &t = sum[d & 1];
+      if (mu == 0) t = SP < 2 ? r : p2_scale_sgn(r, sg);
+      else t = SP < 2 ? p2_add(t, r) : p2_add_sgn(t, r, sg);
+    }
+    acc[c] = p2_add(sum[0], sum[1]);
+  }
+}
+template <bool DAG>
+__device__ __forceinline__ void dwp8_sum(const ulonglong2 (*sm)[kDwp8Threads], int j, int spin, p2 (&acc)[3]) {
+  switch (spin) {
+    case 0: dwp8_spin<DAG, 0>(sm, j, acc); break;
+    case 1: dwp8_spin<DAG, 1>(sm, j, acc); break;
+    case 2: dwp8_spin<DAG, 2>(sm, j, acc); break;
+    default: dwp8_spin<DAG, 3>(sm, j, acc);
   }
 }
 

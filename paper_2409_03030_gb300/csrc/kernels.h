@@ -46,18 +46,13 @@ struct HopParams {
 cudaError_t launch_hop(int prec, const HopParams &P, bool dag, bool axpy, bool norm,
                        cudaStream_t s);
 
-// The double-word hops run two threads per output site on lattices small
-// enough that the two-thread grid fits in one wave of resident blocks (and
-// of at most JQCD_DWP_SPLIT_MAX_VH sites per parity), where one thread per
-// site leaves the GPU short of warps; their grids (and per-block partial
-// sums) are then twice as many blocks.
-#ifndef JQCD_DWP_SPLIT_MAX_VH
-#define JQCD_DWP_SPLIT_MAX_VH 65536
-#endif
-bool dw_hop_split(int64_t vh);
+// The double-word hops run eight threads per output site on small lattices
+// (their grids, and per-block partial sums, are then one per 16 sites), where
+// one thread per site leaves the GPU short of warps.
+bool dw_hop_split8(int64_t vh);
 // Lattices one size up (at most JQCD_DWP_SMALL_MAX_VH sites per parity and a
-// one-thread grid that fits in one wave at a lower occupancy) run one thread
-// per site compiled with a larger register budget.
+// one-thread grid that fits in one wave at a lower occupancy) limit the blocks
+// per SM.
 #ifndef JQCD_DWP_SMALL_MAX_VH
 #define JQCD_DWP_SMALL_MAX_VH 65536
 #endif

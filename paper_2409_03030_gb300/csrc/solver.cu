@@ -14,6 +14,7 @@
 // the tolerance CG restarts from x.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -81,7 +82,7 @@ cudaError_t GaugeEntry::ensure_canon() {
 }
 
 int GaugeEntry::n_partials() const {
-  return 2 * (int)dw_hop_blocks(g.vh) + (int)blas_blocks(24 * g.vh) + 64;
+  return 2 * (int)std::max(dw_hop_blocks(g.vh), hop_blocks(g.vh)) + (int)blas_blocks(24 * g.vh) + 64;
 }
 
 cudaError_t GaugeEntry::ensure_reduce() {

@@ -197,6 +197,41 @@ def test_hop_dw_one_thread_per_site_ragged(jq, dagger, dims):
     g.free()
 
 
+@pytest.mark.parametrize("prec,dims", [(0, (6, 6, 6, 270)), (0, (6, 6, 6, 274))])
+@pytest.mark.parametrize("dagger", [0, 1])
+def test_hop_eight_threads_per_site_edges(jq, dagger, prec, dims):
+    """Hops with eight threads per site, 16-site tiles, at the edges of their
+    rules, with the fused axpy and norm: double-word on 29,160 sites per parity
+    (a ragged last tile) and, past the rule's 29,184, on 29,592.  Against the oracle at sampled sites, the norm against
+    the output's."""
+    jqcd, ctx = jq
+    import torch
+    U = synth.gauge(dims, "expi", eps=0.3, seed=44)
+    g = ctx.gauge_upload(dims, U, t_antiperiodic=True)
+    psi = synth.gaussian_spinor(dims, seed=45)
+    xs = synth.gaussian_spinor(dims, seed=46)
+    pe, po = g.pack(psi, prec)
+    xe, xo = g.pack(xs, prec)
+    norm = torch.zeros(1, dtype=torch.float64, device="cuda")
+    vol = int(np.prod(dims))
+    sites = np.unique(np.concatenate([np.random.default_rng(47).integers(0, vol, 2000), np.arange(64),
+                                      np.arange(vol - 64, vol)]))
+    outs = [g.empty(prec), g.empty(prec)]
+    norms = []
+    for p in (0, 1):
+        g.dslash_eo(prec, p, dagger, po if p == 0 else pe, xe if p == 0 else xo, outs[p], 0.7, -0.12,
+                    norm2=norm)
+        norms.append(norm.item())
+    got = g.unpack(outs[0], outs[1], prec)
+    for p in (0, 1):
+        n_want = np.linalg.norm(only_parity(dims, got, p)) ** 2
+        assert abs(norms[p] - n_want) <= 1e-11 * n_want
+    want = 0.7 * np.transpose(xs.reshape(4, vol, 3)[:, sites], (1, 0, 2)) - 0.12 * oracle.hop_sites(
+        dims, U, psi, sites, dagger=bool(dagger))
+    assert rel(np.transpose(got.reshape(4, vol, 3)[:, sites], (1, 0, 2)), want) <= TOL[prec]
+    g.free()
+
+
 @pytest.mark.parametrize("dims", [(4, 4, 4, 4), (6, 6, 6, 10)])
 @pytest.mark.parametrize("prec", PRECS)
 def test_mdagm_vs_oracle(jq, dims, prec):
