@@ -63,7 +63,6 @@ __global__ void __launch_bounds__(kHopThreads) hop_kernel(const HopParams P) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool active = idx < P.g.vh;
   dwacc nrm{0.f, 0.f};
-  double nrm64 = 0.0;  // FP64 hops accumulate their norm in FP64
   if (active) {
     const HopSite site = hop_site(P.g, (unsigned)idx, P.out_parity);
     C acc[4][3];
@@ -92,13 +91,10 @@ __global__ void __launch_bounds__(kHopThreads) hop_kernel(const HopParams P) {
         for (int c = 0; c < 3; ++c) o[s][c] = T::scale(b, acc[s][c]);
     }
     T::store_spinor(P.out, P.g.vh, idx, o);
-    if (NORM) {
-      if constexpr (PREC == PREC_F64) nrm64 = site_norm2_d(o);
-      else nrm = site_norm2<PREC>(o);
-    }
+    if (NORM) nrm = site_norm2<PREC>(o);
   }
   if (NORM) {
-    const double s = PREC == PREC_F64 ? block_sum_d(nrm64) : block_sum_dw(nrm);
+    const double s = block_sum_dw(nrm);
     if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
     if (P.fin) hop_finish_scalars(P);  // uniform over the grid
   }
@@ -149,17 +145,161 @@ __global__ void __launch_bounds__(kHopThreads, 6) hop_lp_kernel(const HopParams 
   }
 }
 
+// Native FP64 hop with eight threads per output site: a tile is 16 sites in 128
+// threads, warp mu runs direction mu, lanes 0..15 its forward and 16..31 its
+// backward hop.  The kernel is bound by the FP64 pipe (888 FP64 instructions
+// per site), and a warp's FP64 instruction holds its sub-partition's unit for
+// about 67 cycles: with one thread per site a site's 888 last 29 us however
+// few warps there are, and an SM whose unit has one warp more than the others'
+// ends that much later.  In pieces of 111 the work spreads evenly.  The
+// products meet in shared memory; every thread then sums one or two of the
+// 16 x 12 components over the hops, in the order of the one-thread form.
+// Measured on GB300 against one thread per site: 8^4 32.7 -> 6.2 us, 16^4 94.9
+// -> 54.8 us, 16^3x32 127 -> 104 us, 24^3x48 559 -> 517 us (the rate of
+// the FP64 pipe); plain FP64 solve at 16^4 22.9 -> 15.1 ms.
+constexpr int kF64x8Sites = 16;
+constexpr int kF64x8Threads = 8 * kF64x8Sites;
+
+// h = rows 0 and 1 of (1 + S gamma_mu) psi, S = +-1 at run time (riding on the fmas)
+template <int MU>
+__device__ __forceinline__ void project_rt_f64(const cd (&psi)[4][3], cd (&h)[2][3], double S) {
+  typedef SpinTab<MU> T;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const cd q0 = phase<T::p0>(psi[T::j0][c]), q1 = phase<T::p1>(psi[T::j1][c]);
+    h[0][c] = cd{fma(S, q0.re, psi[0][c].re), fma(S, q0.im, psi[0][c].im)};
+    h[1][c] = cd{fma(S, q1.re, psi[1][c].re), fma(S, q1.im, psi[1][c].im)};
+  }
+}
+
+__device__ __forceinline__ double flip_if(double v, bool neg) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
+
+template <bool DAG, bool AXPY, bool NORM>
+__global__ void __launch_bounds__(kF64x8Threads, 4) hop_f64x8_kernel(const HopParams P, int tiles) {
+  __shared__ double2 sm[6][kF64x8Threads];
+  pdl_wait();
+  if (P.guard && *P.guard) return;  // uniform across the grid
+  typedef PT<PREC_F64> T;
+  const Geom &g = P.g;
+  const int p = P.out_parity;
+  const unsigned j = threadIdx.x & 15;
+  double nrm = 0.0;
+  for (int tile = 0; tile < tiles; ++tile) {
+    const unsigned idx = (blockIdx.x * tiles + tile) * kF64x8Sites + j;
+    const bool active = idx < (unsigned)g.vh;
+    if (tile) __syncthreads();  // the last tile's products have been summed
+    if (active) {
+      const int mu = threadIdx.x >> 5;
+      const bool bwd = (threadIdx.x & 16) != 0;
+      const HopSite site = hop_site(g, idx, p);
+      unsigned off;
+      switch (mu) {
+        case 0: off = bwd ? hop_offset(g, site, 1) : hop_offset(g, site, 0); break;
+        case 1: off = bwd ? hop_offset(g, site, 3) : hop_offset(g, site, 2); break;
+        case 2: off = bwd ? hop_offset(g, site, 5) : hop_offset(g, site, 4); break;
+        default: off = bwd ? hop_offset(g, site, 7) : hop_offset(g, site, 6);
+      }
+      const unsigned nb = (off & ~1u) >> 4;
+      cd psi[4][3], h[2][3], u[3][3];
+      T::load_spinor(P.in, g.vh, nb, psi);
+      // W = U_mu(x), or the transpose of U_mu(x - mu), conjugated below
+      const double2 *L = reinterpret_cast<const double2 *>(P.gauge) +
+                         (int64_t)(((bwd ? 1 - p : p) * 4 + mu) * 9) * g.vh + (bwd ? nb : idx);
+      const int sa = bwd ? 1 : 3, sb = bwd ? 3 : 1;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const double2 v = __ldg(L + (int64_t)((k / 3) * sa + (k % 3) * sb) * g.vh);
+        u[k / 3][k % 3] = cd{v.x, flip_if(v.y, bwd)};
+      }
+      const double S = (bwd != DAG) ? 1.0 : -1.0;
+      switch (mu) {
+        case 0: project_rt_f64<0>(psi, h, S); break;
+        case 1: project_rt_f64<1>(psi, h, S); break;
+        case 2: project_rt_f64<2>(psi, h, S); break;
+        default: project_rt_f64<3>(psi, h, S);
+      }
+      T::negate_if(h, off & 1u);
+      cd r[2][3];
+      matvec2<false>(u, h, r);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) sm[k][threadIdx.x] = make_double2(r[k / 3][k % 3].re, r[k / 3][k % 3].im);
+    }
+    if (tile + 1 == tiles) pdl_trigger();
+    __syncthreads();
+    if (active) {
+      const int grp = threadIdx.x >> 4;  // components grp and, for the first four groups, grp + 8
+      const int nk = grp < 4 ? 2 : 1;
+      for (int q = 0; q < nk; ++q) {
+        const int k = grp + 8 * q, spin = k / 3, c = k - 3 * spin;
+        double re = 0.0, im = 0.0;
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+          const int mu = d >> 1;
+          // spins 2 and 3 take the row the projector ties to them, times a phase
+          // (SpinTab; S < 0 negates it)
+          const int src = spin < 2 ? spin : (mu < 2 ? 3 - spin : spin - 2);
+          int ph = 0;
+          if (spin == 2) ph = (mu & 1) ? 0 : 3;
+          if (spin == 3) ph = mu == 0 ? 3 : (mu == 1 ? 2 : (mu == 2 ? 1 : 0));
+          if (spin >= 2 && (((d & 1) != 0) == DAG)) ph ^= 2;
+          const double2 v = sm[3 * src + c][16 * d + j];
+          const bool sw = ph & 1;
+          re += flip_if(sw ? v.y : v.x, ph == 1 || ph == 2);
+          im += flip_if(sw ? v.x : v.y, ph & 2);
+        }
+        cd o;
+        if (AXPY) {
+          const double2 xv = __ldg(reinterpret_cast<const double2 *>(P.x) + (int64_t)k * g.vh + idx);
+          o = T::axpby(P.a, cd{xv.x, xv.y}, P.b, cd{re, im});
+        } else {
+          o = T::scale(P.b, cd{re, im});
+        }
+        reinterpret_cast<double2 *>(P.out)[(int64_t)k * g.vh + idx] = make_double2(o.re, o.im);
+        if (NORM) {
+          nrm = fma(o.re, o.re, nrm);
+          nrm = fma(o.im, o.im, nrm);
+        }
+      }
+    }
+  }
+  if (NORM) {
+    const double s = block_sum_d(nrm);
+    if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
+    if (P.fin) hop_finish_scalars(P);  // uniform over the grid
+  }
+}
+
+// Tiles of 16 sites per block: one while the grid is small, then two, and no
+// more than 16384 blocks (a norm's partial sums, one per block, have that much
+// room in the allocation-free call up to JQCD_NOALLOC_MAX_SITES_PER_PARITY).
+// 24^3x48: 512 us with one tile, 517 with two, 529 with four, 550 with eight;
+// fewer partials keep the solve's sums short.
+static int f64_tiles(int64_t vh) {
+  if (vh <= 65536) return 1;
+  int t = 2;
+  while (vh > (int64_t)16384 * kF64x8Sites * t && t < 64) t *= 2;
+  return t;
+}
+static unsigned f64_blocks(int64_t vh) {
+  const int64_t sites = kF64x8Sites * f64_tiles(vh);
+  return (unsigned)((vh + sites - 1) / sites);
+}
+
 template <int PREC, bool DAG, bool AXPY, bool NORM>
 static cudaError_t launch_hop_t(const HopParams &P, cudaStream_t s) {
-  const unsigned blocks = hop_blocks(P.g.vh);
   note_launch();
-  // FP16: staged (measured faster); FP32: plain loads (its six-chunk stages
-  // cost more occupancy than the prefetch gains); FP64: plain.
-  if (PREC == PREC_F16N)
-    return launch_pdl(hop_lp_kernel<PREC_F16N, DAG, AXPY, NORM>, blocks, kHopThreads,
+  // FP64: eight threads per site.  FP16: staged (measured faster).  FP32: plain
+  // loads (its six-chunk stages cost more occupancy than the prefetch gains).
+  if constexpr (PREC == PREC_F64)
+    return launch_pdl(hop_f64x8_kernel<DAG, AXPY, NORM>, f64_blocks(P.g.vh), kF64x8Threads, 0, s, P,
+                      f64_tiles(P.g.vh));
+  else if constexpr (PREC == PREC_F16N)
+    return launch_pdl(hop_lp_kernel<PREC_F16N, DAG, AXPY, NORM>, hop_blocks(P.g.vh), kHopThreads,
                       lp_stage_smem<PREC_F16N>(), s, P);
   else
-    return launch_pdl(hop_kernel<PREC, DAG, AXPY, NORM>, blocks, kHopThreads, 0, s, P);
+    return launch_pdl(hop_kernel<PREC, DAG, AXPY, NORM>, hop_blocks(P.g.vh), kHopThreads, 0, s, P);
 }
 
 template <int PREC>
@@ -279,6 +419,7 @@ unsigned dw_hop_blocks(int64_t vh) {
 }
 
 unsigned hop_norm_partials(int prec, int64_t vh) {
+  if (prec == PREC_F64) return f64_blocks(vh);
   return prec == PREC_DW ? dw_hop_blocks(vh) : hop_blocks(vh);
 }
 

@@ -82,7 +82,8 @@ cudaError_t GaugeEntry::ensure_canon() {
 }
 
 int GaugeEntry::n_partials() const {
-  return 2 * (int)std::max(dw_hop_blocks(g.vh), hop_blocks(g.vh)) + (int)blas_blocks(24 * g.vh) + 64;
+  const unsigned hop = std::max({dw_hop_blocks(g.vh), hop_norm_partials(PREC_F64, g.vh), hop_blocks(g.vh)});
+  return 2 * (int)hop + (int)blas_blocks(24 * g.vh) + 64;
 }
 
 cudaError_t GaugeEntry::ensure_reduce() {
@@ -371,7 +372,7 @@ double2 *f64_odd(const GaugeEntry &G, double2 *v) { return v + 12 * G.g.vh; }
 // per-block partials of ||out||^2 (2 * hop_blocks entries).
 cudaError_t apply_dirac_f64(const GaugeEntry &G, double kappa, bool dag, double2 *in, double2 *out,
                             double *partials, const int *guard, cudaStream_t s) {
-  const int nb = (int)hop_blocks(G.g.vh);
+  const int nb = (int)hop_norm_partials(PREC_F64, G.g.vh);
   HopParams Pe = G.hop_params(PREC_F64, 0, f64_odd(G, in), f64_even(in), f64_even(out), 1.0,
                               -kappa, partials);
   Pe.guard = guard;
@@ -597,7 +598,7 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
 }
 
 // Plain conjugate gradient in native FP64: every vector, operator and
-// reduction in IEEE double (the hop is hop_kernel<PREC_F64>, the vector
+// reduction in IEEE double (the hop is hop_f64x8_kernel, the vector
 // kernels blas_f64.cu).  Same iteration, stopping rule, true-residual check
 // and restarts as the double-word solver; b in G.fb, x (start vector when
 // use_x0) and the solution in G.fsol, whole lattice in the JQCD_PREC_F64
@@ -610,7 +611,7 @@ static jqcd_status solve_cg_f64(GaugeEntry &G, const jqcd_solve_params &P, cudaS
   const int64_t vh = G.g.vh;
   const int64_t n = (eo ? 12 : 24) * vh;  // complex elements of the system's vectors
   const int nblas = (int)blas_blocks(n);
-  const int nhop = (eo ? 1 : 2) * (int)hop_blocks(vh);
+  const int nhop = (eo ? 1 : 2) * (int)hop_norm_partials(PREC_F64, vh);
   const double tol2 = P.tol * P.tol;
   const double k2 = -P.kappa * P.kappa;
   SolverScalars *S = G.S;

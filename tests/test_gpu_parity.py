@@ -197,12 +197,15 @@ def test_hop_dw_one_thread_per_site_ragged(jq, dagger, dims):
     g.free()
 
 
-@pytest.mark.parametrize("prec,dims", [(0, (6, 6, 6, 270)), (0, (6, 6, 6, 274))])
+@pytest.mark.parametrize("prec,dims", [(0, (6, 6, 6, 270)), (0, (6, 6, 6, 274)), (3, (10, 10, 10, 130)),
+                                       (3, (10, 10, 10, 134)), (3, (32, 32, 32, 34))])
 @pytest.mark.parametrize("dagger", [0, 1])
 def test_hop_eight_threads_per_site_edges(jq, dagger, prec, dims):
     """Hops with eight threads per site, 16-site tiles, at the edges of their
     rules, with the fused axpy and norm: double-word on 29,160 sites per parity
-    (a ragged last tile) and, past the rule's 29,184, on 29,592.  Against the oracle at sampled sites, the norm against
+    (a ragged last tile) and, past the rule's 29,184, on 29,592; FP64 with one
+    tile per block (65,000), two (67,000, a ragged tile in a half-empty block)
+    and four (557,056).  Against the oracle at sampled sites, the norm against
     the output's."""
     jqcd, ctx = jq
     import torch
