@@ -235,6 +235,20 @@ def test_hop_eight_threads_per_site_edges(jq, dagger, prec, dims):
     g.free()
 
 
+def test_current_stream_is_used(jq):
+    """Without a stream argument a call goes to torch's current stream, also
+    inside a stream context; streams, raw handles and buffers are all taken."""
+    jqcd, ctx = jq
+    import torch
+    side = torch.cuda.Stream()
+    for stream in (torch.cuda.current_stream(), side):
+        with torch.cuda.stream(stream):
+            assert jqcd._stream_ptr(None) == stream.cuda_stream
+        assert jqcd._stream_ptr(stream) == jqcd._stream_ptr(stream.cuda_stream) == stream.cuda_stream
+    buf = torch.zeros(16, device="cuda")
+    assert jqcd._dev_ptr(buf) == jqcd._dev_ptr(buf.data_ptr()) == buf.data_ptr()
+
+
 @pytest.mark.parametrize("dims", [(4, 4, 4, 4), (6, 6, 6, 10)])
 @pytest.mark.parametrize("prec", PRECS)
 def test_mdagm_vs_oracle(jq, dims, prec):
