@@ -342,6 +342,47 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS) hop_dwp_ker
   }
 }
 
+// A grid a little over a whole number of one-thread blocks per SM (dw_hop_whole):
+// the first `whole` blocks run 128 sites at one thread each, a multiple of the
+// SM count; eight threads per site share the rest, 16 sites to a block.  The
+// one-thread blocks of such a remainder would each last the whole chain of
+// eight hops, about 7 us, on SMs that are otherwise idle; the tiles last 2.7
+// us.  The trigger comes last (pdl.cuh): the tiles go to the SMs with room.
+template <bool DAG, bool AXPY, bool NORM>
+__global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
+    hop_dwx_kernel(const HopParams P, unsigned whole) {
+  extern __shared__ float4 dsm[];
+  pdl_wait();
+  if (P.guard && *P.guard) return;  // uniform across the grid
+  dwacc nrm{0.f, 0.f};
+  const float4 *const in = reinterpret_cast<const float4 *>(P.in), *const x = reinterpret_cast<const float4 *>(P.x);
+  const float4 *const gauge = reinterpret_cast<const float4 *>(P.gauge);
+  float4 *const out = reinterpret_cast<float4 *>(P.out);
+  if (blockIdx.x < whole) {  // every site of these blocks exists
+    const int64_t idx = (int64_t)blockIdx.x * kDwp1Threads + threadIdx.x;
+    p2 acc[4][3];
+    dwp_hop_site<DAG, kDwp1Threads>(dsm, in, gauge, P.g, P.out_parity, idx, acc);
+    nrm = dwp_store<AXPY, NORM>(acc, out, x, P.g.vh, idx, P.a_split, P.b_split);
+    pdl_trigger();
+  } else {
+    ulonglong2(*sm)[kDwp8Threads] = reinterpret_cast<ulonglong2(*)[kDwp8Threads]>(dsm);
+    const int64_t idx = (int64_t)whole * kDwp1Threads + (int64_t)(blockIdx.x - whole) * kDwp8Sites + (threadIdx.x & 15);
+    if (idx < P.g.vh) dwp8_hop<DAG>(sm, in, gauge, P.g, P.out_parity, (unsigned)idx);
+    pdl_trigger();
+    __syncthreads();
+    const int spin = threadIdx.x >> 4;
+    if (spin < 4 && idx < P.g.vh) {
+      p2 v[3];
+      dwp8_sum<DAG>(sm, threadIdx.x & 15, spin, v);
+      nrm = dwp_store_chunks<AXPY, NORM, 3>(v, 3 * spin, out, x, P.g.vh, idx, P.a_split, P.b_split);
+    }
+  }
+  if (NORM) {
+    const double s = block_sum_dw(nrm);
+    if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
+  }
+}
+
 // Small lattices: eight threads per output site (dwp8_hop).  A hop there is a
 // latency chain, the loads' round trip and the arithmetic of as many hops as a
 // thread runs, on too few warps to hide it: with one hop per thread, 8^4 (two
@@ -373,14 +414,14 @@ __global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS) hop_dwp8_k
   }
 }
 
-// Eight threads per site up to SMs x JQCD_DWP8_BLOCKS blocks of 16 sites
-// (29184 sites per parity).  Measured on GB300, Mhat^dag Mhat p with its norm
-// and the solve, against the two threads per site that ran there before: 8^4
-// 28.9 -> 22.5 us and 1.90 -> 1.58 ms, 12^4 40.9 -> 31.3 us and 2.95 -> 2.55
-// ms, 16^3x12 58.7 -> 52.2 us and 4.18 -> 3.94 ms, 16^3x14 60.1 -> 58.2 us and
-// 4.47 -> 4.41 ms.  One thread per site takes 55.2 us and 4.08 ms at 16^3x12,
-// 55.6 us and 4.32 ms at 16^3x14 (but its sum of eight hops in a row has a 5%
-// larger rounding error), and wins at 16^4 (56.6 against 67.6 us).
+// Eight threads per site up to SMs x JQCD_DWP8_BLOCKS blocks of 16 sites (29184
+// sites per parity).  Measured on GB300 against the two threads per site that
+// ran there before: one hop back to back 8^4 5.3 -> 2.7 us, 12^4 8.3 -> 5.2 us;
+// the double-word solve 8^4 1.90 -> 1.46 ms, 12^4 2.95 -> 2.34 ms, 16^3x12 4.18
+// -> 3.60 ms, 16^3x14 4.47 -> 3.95 ms.  Above, one thread per site solves in
+// less: 16^4 4.44 against 4.53 ms, 16^3x18 4.62 against 5.14 ms, 16^3x24 5.88
+// against 6.75 ms.  Four blocks per SM: with five (96 registers, 40 bytes
+// spilled) 8^4 takes 2.9 us, with three 12^4 5.6 us.
 bool dw_hop_split8(int64_t vh) {
   static const int64_t max_vh = [] {
     int dev = 0, sms = 0;
@@ -413,8 +454,33 @@ bool dw_hop_small(int64_t vh) {
   return !dw_hop_split8(vh) && vh <= max_vh && vh <= JQCD_DWP_SMALL_MAX_VH;
 }
 
+// Whole blocks per SM at one thread per site and the rest at eight, where the
+// rest is at most two fifths of a block per SM: one hop on GB300 against one
+// thread for every site: 16^3x30 21.9 -> 18.1 us, 16^3x32 22.1 -> 19.8 us,
+// 16^3x40 27.6 -> 25.1 us, 16^3x48 33.4 -> 29.9 us, 20^3x40 49.1 -> 47.5 us;
+// the double-word solve at 20x18x14x26 8.25 -> 7.82 ms.  With a longer rest the
+// tiles last longer than the blocks they replace (20^3x24, 0.93 of a block per
+// SM: 29.5 -> 32.0 us), and past JQCD_DWX_MAX_VH a rest no longer shows (24^3x48
+// 91.0 and 90.9 us; the solve at 24^3x32 21.9 and 22.1 ms).  Not below one
+// wave of one-thread blocks (16^3x24: 16.9 -> 17.1 us, 16^3x28 17.1 -> 19.3 us).
+unsigned dw_hop_whole(int64_t vh) {
+  static const int64_t sms = [] {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
+      return (int64_t)0;
+    return (int64_t)n;
+  }();
+  const int64_t wave = sms * JQCD_DWP_MIN_BLOCKS * kDwp1Threads;
+  if (!sms || vh <= wave || vh > JQCD_DWX_MAX_VH) return 0;
+  const int64_t blocks = (vh + kDwp1Threads - 1) / kDwp1Threads, whole = vh / kDwp1Threads / sms * sms;
+  return 5 * (blocks - whole) <= 2 * sms ? (unsigned)whole : 0;
+}
+
 unsigned dw_hop_blocks(int64_t vh) {
-  if (dw_hop_split8(vh)) return (unsigned)((vh + kDwp8Sites - 1) / kDwp8Sites);
+  const int64_t whole = dw_hop_whole(vh);
+  if (whole || dw_hop_split8(vh))
+    return (unsigned)(whole + (vh - whole * kDwp1Threads + kDwp8Sites - 1) / kDwp8Sites);
   return (unsigned)((vh + kDwp1Threads - 1) / kDwp1Threads);
 }
 
@@ -427,17 +493,22 @@ template <bool DAG, bool AXPY, bool NORM>
 static cudaError_t launch_hop_dw_t(const HopParams &P, cudaStream_t s) {
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
-  auto kern = hop_dwp_kernel<DAG, AXPY, NORM>;
   if (!configured) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
+    cudaError_t e = cudaFuncSetAttribute(hop_dwp_kernel<DAG, AXPY, NORM>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(hop_dwx_kernel<DAG, AXPY, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kDwp1Smem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
+  const unsigned blocks = dw_hop_blocks(P.g.vh);
   if (dw_hop_split8(P.g.vh))
-    return launch_pdl(hop_dwp8_kernel<DAG, AXPY, NORM>, dw_hop_blocks(P.g.vh), kDwp8Threads, 0, s, P);
-  return launch_pdl(kern, dw_hop_blocks(P.g.vh), kDwp1Threads, dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s,
-                    P);
+    return launch_pdl(hop_dwp8_kernel<DAG, AXPY, NORM>, blocks, kDwp8Threads, 0, s, P);
+  if (const unsigned whole = dw_hop_whole(P.g.vh))
+    return launch_pdl(hop_dwx_kernel<DAG, AXPY, NORM>, blocks, kDwp1Threads, kDwp1Smem, s, P, whole);
+  return launch_pdl(hop_dwp_kernel<DAG, AXPY, NORM>, blocks, kDwp1Threads,
+                    dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P);
 }
 
 static cudaError_t launch_hop_dw(const HopParams &P, bool dag, bool axpy, bool norm, cudaStream_t s) {

@@ -92,6 +92,43 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
   if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
 }
 
+// The same with the sites of `whole` blocks at one thread each and eight
+// threads for each of the others (dw_hop_whole).
+template <bool XUPD>
+__global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
+    hop_dwx_cg_kernel(const HopParams P, unsigned whole, const float4 *__restrict__ p, float4 *__restrict__ xs,
+                      const float4 *r_in, float4 *r, const float2 *__restrict__ alpha) {
+  extern __shared__ float4 dsm[];
+  pdl_wait();
+  if (P.guard && *P.guard) return;  // uniform across the grid
+  dwacc nrm{0.f, 0.f};
+  const float4 *const in = reinterpret_cast<const float4 *>(P.in), *const x = reinterpret_cast<const float4 *>(P.x);
+  const float4 *const gauge = reinterpret_cast<const float4 *>(P.gauge);
+  if (blockIdx.x < whole) {  // every site of these blocks exists
+    const int64_t idx = (int64_t)blockIdx.x * kDwp1Threads + threadIdx.x;
+    p2 acc[4][3], v[12];
+    dwp_hop_site<true, kDwp1Threads>(dsm, in, gauge, P.g, P.out_parity, idx, acc);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = acc[k / 3][k % 3];
+    nrm = dwp_store_cg<XUPD, 12>(v, 0, x, p, xs, r_in, r, P.g.vh, idx, P.a_split, P.b_split, *alpha);
+    pdl_trigger();
+  } else {
+    ulonglong2(*sm)[kDwp8Threads] = reinterpret_cast<ulonglong2(*)[kDwp8Threads]>(dsm);
+    const int64_t idx = (int64_t)whole * kDwp1Threads + (int64_t)(blockIdx.x - whole) * kDwp8Sites + (threadIdx.x & 15);
+    if (idx < P.g.vh) dwp8_hop<true>(sm, in, gauge, P.g, P.out_parity, (unsigned)idx);
+    pdl_trigger();
+    __syncthreads();
+    const int spin = threadIdx.x >> 4;
+    if (spin < 4 && idx < P.g.vh) {
+      p2 v[3];
+      dwp8_sum<true>(sm, threadIdx.x & 15, spin, v);
+      nrm = dwp_store_cg<XUPD, 3>(v, 3 * spin, x, p, xs, r_in, r, P.g.vh, idx, P.a_split, P.b_split, *alpha);
+    }
+  }
+  const double s = block_sum_dw(nrm);
+  if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
+}
+
 // The same with eight threads per output site (small lattices, dw_hop_split8).
 template <bool XUPD>
 __global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS)
@@ -178,14 +215,20 @@ static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x
   note_launch();
   static bool configured = false;  // one attribute call per instantiation
   if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        hop_dwp_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
+    cudaError_t e = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kDwpSmallSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(hop_dwx_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kDwp1Smem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
+  const unsigned blocks = dw_hop_blocks(P.g.vh);
   if (dw_hop_split8(P.g.vh))
-    return launch_pdl(hop_dwp8_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp8Threads, 0, s, P, p, x, r_in, r, alpha);
-  return launch_pdl(hop_dwp_cg_kernel<XUPD>, dw_hop_blocks(P.g.vh), kDwp1Threads,
+    return launch_pdl(hop_dwp8_cg_kernel<XUPD>, blocks, kDwp8Threads, 0, s, P, p, x, r_in, r, alpha);
+  if (const unsigned whole = dw_hop_whole(P.g.vh))
+    return launch_pdl(hop_dwx_cg_kernel<XUPD>, blocks, kDwp1Threads, kDwp1Smem, s, P, whole, p, x, r_in, r, alpha);
+  return launch_pdl(hop_dwp_cg_kernel<XUPD>, blocks, kDwp1Threads,
                     dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P, p, x, r_in, r, alpha);
 }
 

@@ -330,8 +330,9 @@ __device__ __forceinline__ void dwp_hop_site(float4 *dsm, const float4 *in, cons
 // lanes 0..15 the forward and 16..31 the backward hop of sites 0..15.  Each
 // thread loads its operands straight into registers (one round trip for all
 // of them), leaves its two-spin product in shared memory, and the first
-// 4 x kDwp8Sites threads sum one spin of one site each (dwp8_spin).  A hop's
-// latency chain is then one hop long.
+// 4 x kDwp8Sites threads sum one spin of one site each (dwp8_spin; with a branch
+// per half-warp instead of one stream for both spins 12^4 took 6.0 us, not
+// 5.2).  A hop's latency chain is then one hop long.
 constexpr int kDwp8Sites = 16;
 constexpr int kDwp8Threads = 8 * kDwp8Sites;
 
@@ -393,46 +394,41 @@ __device__ __forceinline__ void dwp8_hop(ulonglong2 (*sm)[kDwp8Threads], const f
   }
 }
 
-// acc = spin SP of (H in) at site j of the block: the forward and the backward
+// acc = spin 2 HI + s of (H in) at site j of the tile (HI by warp, s = 0 or 1 by
+// half-warp, one instruction stream for both): the forward and the backward
 // hops' sums, added (shorter chains than all eight in a row, and on average a
-// smaller rounding error: 6.41e-14 against 6.76e-14 at 12^4).
-// The terms are those of reconstruct_half_p; the first of each sum is taken as
-// it is.
-template <bool DAG, int SP>
-__device__ __forceinline__ void dwp8_spin(const ulonglong2 (*sm)[kDwp8Threads], int j, p2 (&acc)[3]) {
+// smaller rounding error: 6.41e-14 against 6.76e-14 at 12^4).  The terms are
+// those of reconstruct_half_p; the first of each sum is taken as it is.
+template <bool DAG, int HI>
+__device__ __forceinline__ void dwp8_spin(const ulonglong2 (*sm)[kDwp8Threads], int j, int s, p2 (&acc)[3]) {
+  const f2 flip = s ? 0x8000000080000000ull : 0ull;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     p2 sum[2];
 #pragma unroll
-    for (int d = 0; d < 8; ++d) {  // everything but the data is constant after unrolling
+    for (int d = 0; d < 8; ++d) {  // everything but the data and s is constant after unrolling
       const int mu = d >> 1;
-      const int src = SP < 2 ? SP : (mu < 2 ? 3 - SP : SP - 2);
-      const ulonglong2 v = sm[3 * src + c][16 * d + j];
+      const ulonglong2 v = sm[3 * (HI && mu < 2 ? 1 - s : s) + c][16 * d + j];
       p2 r{v.x, v.y};
-      f2 sg = f2_make(1.f, 1.f);
-      if (SP >= 2) {
-        const float S = (((d & 1) != 0) != DAG) ? 1.f : -1.f;
-        if (!(mu & 1)) r = p2_swap(r);
-        if (mu == 0 || (mu == 2 && SP == 2)) sg = f2_make(S, -S);
-        if (mu == 2 && SP == 3) sg = f2_make(-S, S);
-        if (mu == 3 || (mu == 1 && SP == 2)) sg = f2_make(S, S);
-        if (mu == 1 && SP == 3) sg = f2_make(-S, -S);
-      }
       p2 &t = sum[d & 1];
-      if (mu == 0) t = SP < 2 ? r : p2_scale_sgn(r, sg);
-      else t = SP < 2 ? p2_add(t, r) : p2_add_sgn(t, r, sg);
+      if (HI) {
+        const float S = (((d & 1) != 0) != DAG) ? 1.f : -1.f;
+        f2 sg = f2_make(S, (mu & 1) ? S : -S);
+        if (mu == 1 || mu == 2) sg ^= flip;
+        if (!(mu & 1)) r = p2_swap(r);
+        t = mu == 0 ? p2_scale_sgn(r, sg) : p2_add_sgn(t, r, sg);
+      } else {
+        t = mu == 0 ? r : p2_add(t, r);
+      }
     }
     acc[c] = p2_add(sum[0], sum[1]);
   }
 }
+// The same by run-time spin = 0..3, uniform over each pair of half-warps.
 template <bool DAG>
 __device__ __forceinline__ void dwp8_sum(const ulonglong2 (*sm)[kDwp8Threads], int j, int spin, p2 (&acc)[3]) {
-  switch (spin) {
-    case 0: dwp8_spin<DAG, 0>(sm, j, acc); break;
-    case 1: dwp8_spin<DAG, 1>(sm, j, acc); break;
-    case 2: dwp8_spin<DAG, 2>(sm, j, acc); break;
-    default: dwp8_spin<DAG, 3>(sm, j, acc);
-  }
+  if (spin >> 1) dwp8_spin<DAG, 1>(sm, j, spin & 1, acc);
+  else dwp8_spin<DAG, 0>(sm, j, spin & 1, acc);
 }
 
 // out = a x + b v (AXPY) or b v for NC consecutive components k0 .. k0 + NC - 1

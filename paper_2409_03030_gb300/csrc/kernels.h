@@ -57,6 +57,12 @@ bool dw_hop_split8(int64_t vh);
 #define JQCD_DWP_SMALL_MAX_VH 65536
 #endif
 bool dw_hop_small(int64_t vh);
+// Whole blocks of 128 sites, one thread each, of a launch that gives its other
+// sites eight threads each (0: all sites are handled alike).
+#ifndef JQCD_DWX_MAX_VH
+#define JQCD_DWX_MAX_VH 163840
+#endif
+unsigned dw_hop_whole(int64_t vh);
 unsigned dw_hop_blocks(int64_t vh);                 // blocks of a double-word hop launch
 unsigned hop_norm_partials(int prec, int64_t vh);   // partials of a hop launch with norm
 

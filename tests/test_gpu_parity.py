@@ -197,13 +197,16 @@ def test_hop_dw_one_thread_per_site_ragged(jq, dagger, dims):
     g.free()
 
 
-@pytest.mark.parametrize("prec,dims", [(0, (6, 6, 6, 270)), (0, (6, 6, 6, 274)), (3, (10, 10, 10, 130)),
+@pytest.mark.parametrize("prec,dims", [(0, (6, 6, 6, 270)), (0, (6, 6, 6, 274)), (0, (6, 6, 6, 540)),
+                                       (0, (6, 6, 6, 542)), (0, (20, 18, 14, 26)), (3, (10, 10, 10, 130)),
                                        (3, (10, 10, 10, 134)), (3, (32, 32, 32, 34))])
 @pytest.mark.parametrize("dagger", [0, 1])
 def test_hop_eight_threads_per_site_edges(jq, dagger, prec, dims):
     """Hops with eight threads per site, 16-site tiles, at the edges of their
     rules, with the fused axpy and norm: double-word on 29,160 sites per parity
-    (a ragged last tile) and, past the rule's 29,184, on 29,592; FP64 with one
+    (a ragged last tile) and, past the rule's 29,184, on 29,592; around one wave
+    of one-thread blocks (58,368 sites), past which eight threads per site take
+    the rest, on 58,320, 58,536 (a rest of 168 sites) and 65,520; FP64 with one
     tile per block (65,000), two (67,000, a ragged tile in a half-empty block)
     and four (557,056).  Against the oracle at sampled sites, the norm against
     the output's."""
@@ -406,6 +409,21 @@ def test_mixed_cg_16x4(jq, mode):
     assert err <= bound, (err, bound)
     xd, info_d, st_d = g.cg_solve(b, 0.12, tol=1e-10, eo=True, mode=jqcd.CG_DW)
     assert rel(x, xd) < 1e-7
+    g.free()
+
+
+@pytest.mark.parametrize("dims", [(6, 6, 6, 270), (6, 6, 6, 542)])
+def test_cg_dw_eight_threads_per_site(jq, dims):
+    """The double-word CG's fused last hop with a ragged tile: eight threads for
+    every site, and for the rest of a grid of whole blocks."""
+    jqcd, ctx = jq
+    U = synth.gauge(dims, "expi", eps=0.3, seed=48)
+    b = synth.gaussian_spinor(dims, seed=49)
+    g = ctx.gauge_upload(dims, U)
+    x, info, st = g.cg_solve(b, 0.12, tol=1e-10, mode=jqcd.CG_DW)
+    assert st == 0
+    res = system_residual(dims, U, b, x, 0.12, True)
+    assert res <= 1e-10 * (1 + 1e-6), res
     g.free()
 
 
