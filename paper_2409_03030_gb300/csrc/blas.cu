@@ -115,16 +115,18 @@ __global__ void finalize_sum_kernel(const double *partials, int n, double *out) 
 
 __global__ void cg_alpha_kernel(const double *partials, int n, SolverScalars *S, int x_code) {
   pdl_enter();
-  if (S->halt) return;
+  const int halt = S->halt;
+  const double rr = S->rr;
   const double pAp = block_sum_partials(partials, n);
-  if (threadIdx.x == 0) cg_alpha_step(pAp, S, x_code);
+  if (threadIdx.x == 0 && !halt) cg_alpha_step(pAp, rr, S, x_code);
 }
 
 __global__ void cg_beta_kernel(const double *partials, int n, SolverScalars *S) {
   pdl_enter();
-  if (S->halt) return;
+  const int halt = S->halt;
+  const ScalarsIn in = scalars_in(S);
   const double rr_new = block_sum_partials(partials, n);
-  if (threadIdx.x == 0) cg_beta_step(rr_new, S);
+  if (threadIdx.x == 0 && !halt) cg_beta_step(rr_new, in, S);
 }
 
 __global__ void cg_start_kernel(const double *partials, int n, SolverScalars *S, double tol2,
@@ -146,7 +148,7 @@ __global__ void cg_start_kernel(const double *partials, int n, SolverScalars *S,
 
 cudaError_t launch_finalize_sum(const double *partials, int n, double *out, cudaStream_t s) {
   note_launch();
-  return launch_pdl(finalize_sum_kernel, 1, kReduceThreads, 0, s, partials, n, out);
+  return launch_pdl(finalize_sum_kernel, 1, reduce_threads(n), 0, s, partials, n, out);
 }
 cudaError_t launch_dw_copy(float4 *dst, const float4 *src, int64_t n, cudaStream_t s) {
   note_launch();
@@ -182,16 +184,16 @@ cudaError_t launch_dw_xpay(float4 *p, const float4 *r, int64_t n, const SolverSc
 }
 cudaError_t launch_cg_alpha(const double *partials, int n, SolverScalars *S, cudaStream_t s, int x_code) {
   note_launch();
-  return launch_pdl(cg_alpha_kernel, 1, kReduceThreads, 0, s, partials, n, S, x_code);
+  return launch_pdl(cg_alpha_kernel, 1, reduce_threads(n), 0, s, partials, n, S, x_code);
 }
 cudaError_t launch_cg_beta(const double *partials, int n, SolverScalars *S, cudaStream_t s) {
   note_launch();
-  return launch_pdl(cg_beta_kernel, 1, kReduceThreads, 0, s, partials, n, S);
+  return launch_pdl(cg_beta_kernel, 1, reduce_threads(n), 0, s, partials, n, S);
 }
 cudaError_t launch_cg_start(const double *partials, int n, SolverScalars *S, double tol2,
                             int max_iters, double delta2, cudaStream_t s) {
   note_launch();
-  cg_start_kernel<<<1, kReduceThreads, 0, s>>>(partials, n, S, tol2, max_iters, delta2);
+  cg_start_kernel<<<1, reduce_threads(n), 0, s>>>(partials, n, S, tol2, max_iters, delta2);
   return cudaGetLastError();
 }
 

@@ -125,9 +125,10 @@ __global__ void dw_add_f32_kernel(float4 *__restrict__ x, float4 *__restrict__ x
 
 __global__ void mixed_beta_kernel(const double *partials, int n, SolverScalars *S) {
   pdl_enter();
-  if (S->halt) return;
+  const int halt = S->halt;
+  const ScalarsIn in = scalars_in(S);
   const double rr_new = block_sum_partials(partials, n);
-  if (threadIdx.x == 0) mixed_beta_step(rr_new, S);
+  if (threadIdx.x == 0 && !halt) mixed_beta_step(rr_new, in, S);
 }
 
 __global__ void mixed_after_update_kernel(const double *partials, int n, SolverScalars *S) {
@@ -192,13 +193,13 @@ cudaError_t launch_dw_add_f32(float4 *x, float4 *xs, int64_t vh, cudaStream_t s)
 
 cudaError_t launch_mixed_beta(const double *partials, int n, SolverScalars *S, cudaStream_t s) {
   note_launch();
-  return launch_pdl(mixed_beta_kernel, 1, kReduceThreads, 0, s, partials, n, S);
+  return launch_pdl(mixed_beta_kernel, 1, reduce_threads(n), 0, s, partials, n, S);
 }
 
 cudaError_t launch_mixed_after_update(const double *partials, int n, SolverScalars *S,
                                       cudaStream_t s) {
   note_launch();
-  mixed_after_update_kernel<<<1, kReduceThreads, 0, s>>>(partials, n, S);
+  mixed_after_update_kernel<<<1, reduce_threads(n), 0, s>>>(partials, n, S);
   return cudaGetLastError();
 }
 

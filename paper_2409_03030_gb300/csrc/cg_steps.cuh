@@ -19,93 +19,86 @@ __device__ __forceinline__ float2 split_double(double v) {
   return make_float2(h, __double2float_rn(v - (double)h));
 }
 
+// What the scalar steps read of S, loaded before the partials are summed so that
+// its latency runs beside theirs.
+struct ScalarsIn {
+  double rr, stop_rr, delta2, rr_max;
+  int iters, max_iters;
+};
+__device__ __forceinline__ ScalarsIn scalars_in(const SolverScalars *S) {
+  return ScalarsIn{S->rr, S->stop_rr, S->delta2, S->rr_max, S->iters, S->max_iters};
+}
+
 // alpha = rr / pAp; a non-positive or non-finite pAp ends the solve (breakdown).
 // x_code != 0: step (x_code & 15) - 1 of block x_code >> 4 of the inner
 // iterations; its alpha is recorded for the block's update of x_s.
-__device__ __forceinline__ void cg_alpha_step(double pAp, SolverScalars *S, int x_code) {
+__device__ __forceinline__ void cg_alpha_step(double pAp, double rr, SolverScalars *S, int x_code) {
   S->pAp = pAp;
   if (!(pAp > 0.0) || !isfinite(pAp)) {
     S->done = 2;
     S->halt = 1;
     return;
   }
-  const double a = S->rr / pAp;
+  const double a = rr / pAp;
   S->alpha = a;
-  S->alpha_dw = split_double(a);
-  S->malpha_dw = split_double(-a);
-  S->alpha_f = (float)a;
-  S->malpha_f = (float)-a;
+  const float2 d = split_double(a);  // d.x = (float)a
+  S->alpha_dw = d;
+  S->malpha_dw = make_float2(-d.x, -d.y);
+  S->alpha_f = d.x;
+  S->malpha_f = -d.x;
   if (x_code) {
-    S->alpha_h[(x_code & 15) - 1] = (float)a;
+    S->alpha_h[(x_code & 15) - 1] = d.x;
     S->x_code = x_code;
   }
 }
 
 // beta = rr_new / rr, the stopping test on rr_new and the iteration cap
-__device__ __forceinline__ void cg_beta_step(double rr_new, SolverScalars *S) {
+__device__ __forceinline__ void cg_beta_step(double rr_new, const ScalarsIn &I, SolverScalars *S) {
   S->rr_new = rr_new;
-  S->iters += 1;
+  S->iters = I.iters + 1;
   if (!isfinite(rr_new)) {
     S->done = 2;
     S->halt = 1;
     return;
   }
-  if (rr_new <= S->stop_rr) {
-    S->rr = rr_new;
+  S->rr = rr_new;
+  if (rr_new <= I.stop_rr) {
     S->done = 1;
     S->halt = 1;
     return;
   }
-  if (S->iters >= S->max_iters) {
+  if (I.iters + 1 >= I.max_iters) {
     S->done = 3;
     S->halt = 1;
   }
-  const double b = rr_new / S->rr;
+  const double b = rr_new / I.rr;
   S->beta = b;
-  S->beta_dw = split_double(b);
-  S->beta_f = (float)b;
-  S->rr = rr_new;
+  const float2 d = split_double(b);
+  S->beta_dw = d;
+  S->beta_f = d.x;
 }
 
 // The inner solver of the mixed-precision CG: the same beta, and a reliable
 // update requested (need_update, halt) when rr_new reaches the tolerance,
 // drops below delta^2 max ||r||^2 since the last update, or at the cap.
-__device__ __forceinline__ void mixed_beta_step(double rr_new, SolverScalars *S) {
+__device__ __forceinline__ void mixed_beta_step(double rr_new, const ScalarsIn &I, SolverScalars *S) {
   S->rr_new = rr_new;
-  S->iters += 1;
+  S->iters = I.iters + 1;
   if (!isfinite(rr_new)) {
     S->done = 2;
     S->halt = 1;
     return;
   }
-  if (rr_new <= S->stop_rr || rr_new < S->delta2 * S->rr_max || S->iters >= S->max_iters) {
+  if (rr_new <= I.stop_rr || rr_new < I.delta2 * I.rr_max || I.iters + 1 >= I.max_iters) {
     S->need_update = 1;  // the host runs the double-word update next
     S->halt = 1;
     return;
   }
-  const double b = rr_new / S->rr;
+  const double b = rr_new / I.rr;
   S->beta = b;
   S->beta_f = (float)b;
   S->rr = rr_new;
-  if (rr_new > S->rr_max) S->rr_max = rr_new;
-}
-
-// block_sum_partials with its loads from L2 (ld.global.cg): the partials
-// were written by other blocks of the same launch.
-__device__ __forceinline__ double block_sum_partials_l2(const double *partials, int n) {
-  double v = 0.0;
-  constexpr int kU = 16;
-  for (int base = threadIdx.x; base < n; base += kU * blockDim.x) {
-    double t[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = base + u * (int)blockDim.x;
-      t[u] = i < n ? __ldcg(partials + i) : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v += t[u];
-  }
-  return block_sum_d(v);
+  if (rr_new > I.rr_max) S->rr_max = rr_new;
 }
 
 // Called by every thread of every block of a hop launch after thread 0 has
@@ -124,12 +117,13 @@ __device__ __forceinline__ void hop_finish_scalars(const HopParams &P) {
   __syncthreads();
   if (!is_last) return;  // uniform over the block
   __threadfence();
-  const double v = block_sum_partials_l2(P.partials, (int)gridDim.x);
+  SolverScalars *S = P.fin_S;
+  const ScalarsIn in = scalars_in(S);
+  const double v = block_sum_partials<true>(P.partials, (int)gridDim.x);
   if (threadIdx.x == 0) {
-    SolverScalars *S = P.fin_S;
     S->fin_count = 0;
-    if (P.fin == FIN_ALPHA) cg_alpha_step(v, S, P.x_code);
-    else mixed_beta_step(v, S);
+    if (P.fin == FIN_ALPHA) cg_alpha_step(v, in.rr, S, P.x_code);
+    else mixed_beta_step(v, in, S);
   }
 }
 

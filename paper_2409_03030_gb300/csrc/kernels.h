@@ -80,6 +80,10 @@ cudaError_t launch_spinor_unpack(const Geom &g, int prec, const void *even, cons
 // ---- BLAS-1 and reductions ---------------------------------------------------
 constexpr int kBlasThreads = 256;
 constexpr int kReduceThreads = 256;
+// Threads of a single-block sum of n partials: one warp per FP64 unit while
+// sixteen loads a thread bring all of them in one batch, more where a second
+// batch's latency costs more than the extra warps' adds.
+inline int reduce_threads(int n) { return n <= 2048 ? 128 : (n <= 4096 ? 256 : 512); }
 unsigned blas_blocks(int64_t n);   // grid of the grid-stride vector kernels
 
 // Device-resident solver scalars.

@@ -47,26 +47,8 @@ __device__ __forceinline__ dw dw_from_double(double v) {
   return dw_make(h, __double2float_rn(v - (double)h));
 }
 
-__device__ __forceinline__ double sum_partials(const double *partials, int n) {
-  double v = 0.0;
-  // all of a thread's loads are in flight before its first add; the adds keep
-  // the fixed order i = tid, tid + blockDim.x, ... (out-of-range slots add 0)
-  constexpr int kU = 16;
-  for (int base = threadIdx.x; base < n; base += kU * blockDim.x) {
-    double t[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = base + u * (int)blockDim.x;
-      t[u] = i < n ? partials[i] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v += t[u];
-  }
-  return block_sum_d(v);
-}
-
 __global__ void ms_start_kernel(const double *partials, int n, MsScalars *S, double tol2, int max_iters) {
-  const double rhs2 = sum_partials(partials, n);
+  const double rhs2 = block_sum_partials(partials, n);
   if (threadIdx.x == 0) {
     S->rhs2 = rhs2;
     S->rr = rhs2;
@@ -98,20 +80,25 @@ __global__ void ms_alpha_kernel(const double *partials, int n, MsScalars *S, MsS
   __shared__ double sh_pap;
   pdl_enter();
   if (slot == 0 && threadIdx.x == 0) B->n = 0;  // the last record has been applied
-  if (S->halt) return;
-  const double v = sum_partials(partials, n);
+  const int i = threadIdx.x;
+  const bool mine = i < S->nshift;
+  // what the step reads, loaded beside the partials
+  const int halt = S->halt, act = mine ? S->active[i] : 0;
+  const double rr = S->rr, ap = S->alpha_prev, b = S->beta;
+  const double z = mine ? S->zeta[i] : 1.0, zp = mine ? S->zeta_prev[i] : 1.0, sigma = mine ? S->sigma[i] : 0.0;
+  const double v = block_sum_partials(partials, n);
+  if (halt) return;
   if (threadIdx.x == 0) sh_pap = v;
   __syncthreads();
+  if (i > 0 && !act) return;
   const double pAp = sh_pap;
   if (!(pAp > 0.0) || !isfinite(pAp)) {
     if (threadIdx.x == 0) { S->done = 2; S->halt = 1; }
     return;
   }
-  const double a = S->rr / pAp, ap = S->alpha_prev, b = S->beta;
-  const int i = threadIdx.x;
-  if (i < S->nshift && S->active[i]) {
-    const double z = S->zeta[i], zp = S->zeta_prev[i];
-    const double zn = z * zp * ap / (a * b * (zp - z) + zp * ap * (1.0 + S->sigma[i] * a));
+  const double a = rr / pAp;
+  if (act) {
+    const double zn = z * zp * ap / (a * b * (zp - z) + zp * ap * (1.0 + sigma * a));
     S->zeta_next[i] = zn;
     S->alpha_s[i] = a * zn / z;
   }
@@ -130,28 +117,30 @@ __device__ __forceinline__ float2 split_pair(double v) {
 __global__ void ms_beta_kernel(const double *partials, int n, MsScalars *S, MsSteps *B, int slot) {
   __shared__ double sh_rr;
   pdl_enter();
-  if (S->halt) return;
-  const double v = sum_partials(partials, n);
+  const int i = threadIdx.x;
+  const bool mine = i < S->nshift;
+  // what the step reads, loaded beside the partials
+  const int halt = S->halt, iter = S->iters + 1;
+  const bool last = iter >= S->max_iters, act = mine && S->active[i] != 0;
+  const double rr = S->rr, stop_rr = S->stop_rr;
+  const double z = mine ? S->zeta[i] : 1.0, zn = mine ? S->zeta_next[i] : 1.0, as = mine ? S->alpha_s[i] : 0.0;
+  const double v = block_sum_partials(partials, n);
+  if (halt) return;
   if (threadIdx.x == 0) sh_rr = v;
   __syncthreads();
   const double rr_new = sh_rr;
-  const int iter = S->iters + 1;
-  const bool last = iter >= S->max_iters;
   const bool finite = isfinite(rr_new);
-  const double b = rr_new / S->rr;
-  const int i = threadIdx.x;
+  const double b = mine || i == 0 ? rr_new / rr : 0.0;
   int running = 0;  // this thread's shift goes on
-  if (finite && i < S->nshift) {
-    const bool act = S->active[i] != 0;
+  if (finite && mine) {
     float2 al = make_float2(0.f, 0.f), ze = al, be = al;
     if (act) {
-      const double z = S->zeta[i], zn = S->zeta_next[i];
-      al = split_pair(S->alpha_s[i]);
+      al = split_pair(as);
       ze = split_pair(zn);
       be = split_pair(b * (zn / z) * (zn / z));
       S->zeta_prev[i] = z;
       S->zeta[i] = zn;
-      if (zn * zn * rr_new <= S->stop_rr) {
+      if (zn * zn * rr_new <= stop_rr) {
         S->active[i] = 0;
         S->conv_iter[i] = iter;
       } else {
@@ -444,19 +433,19 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
 cudaError_t launch_ms_start(const double *partials, int n, MsScalars *S, double tol2, int max_iters,
                             cudaStream_t s) {
   note_launch();
-  ms_start_kernel<<<1, kReduceThreads, 0, s>>>(partials, n, S, tol2, max_iters);
+  ms_start_kernel<<<1, reduce_threads(n), 0, s>>>(partials, n, S, tol2, max_iters);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ms_alpha(const double *partials, int nhop, MsScalars *S, MsSteps *B, int slot, cudaStream_t s) {
   note_launch();
-  return launch_pdl(ms_alpha_kernel, 1, kReduceThreads, 0, s, partials, nhop, S, B, slot);
+  return launch_pdl(ms_alpha_kernel, 1, reduce_threads(nhop), 0, s, partials, nhop, S, B, slot);
 }
 
 cudaError_t launch_ms_beta_p(const double *partials, int nhop, int nblas, MsScalars *S, MsSteps *B, int slot,
                              const float4 *r, float4 *pb, int64_t n, cudaStream_t s) {
   note_launch(2);
-  const cudaError_t e = launch_pdl(ms_beta_kernel, 1, kReduceThreads, 0, s, partials, nhop, S, B, slot);
+  const cudaError_t e = launch_pdl(ms_beta_kernel, 1, reduce_threads(nhop), 0, s, partials, nhop, S, B, slot);
   if (e != cudaSuccess) return e;
   return launch_pdl(ms_p_kernel, nblas, kBlasThreads, 0, s, pb, r, n, S);
 }

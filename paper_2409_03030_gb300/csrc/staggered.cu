@@ -265,46 +265,27 @@ __global__ void stag_xpay_norm_kernel(float4 *__restrict__ p, const float4 *__re
 // alpha = ||r||^2 / <p, (m^2 - D_eo D_oe) p> with <p, A p> = m^2 ||p||^2 + ||D_oe p||^2
 // (D_eo^dag = -D_oe): the two norms come as per-block partials of the first
 // hop (pt) and of the p update (pp); breakdown when the sum is not positive.
-// This thread's share of sum(a[0..n)) in the fixed order i = tid, tid +
-// blockDim.x, ...; all of its loads are in flight before its first add
-// (out-of-range slots add 0).
-__device__ __forceinline__ double thread_sum(const double *a, int n) {
-  constexpr int kU = 16;
-  double v = 0.0;
-  for (int base = threadIdx.x; base < n; base += kU * blockDim.x) {
-    double t[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = base + u * (int)blockDim.x;
-      t[u] = i < n ? a[i] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) v += t[u];
-  }
-  return v;
-}
-
 __global__ void stag_alpha_kernel(const double *pt, int nt, const double *pp, int np, double m2,
                                   SolverScalars *S) {
   pdl_enter();
-  if (S->halt) return;
-  double vt = thread_sum(pt, nt), vp = thread_sum(pp, np);
-  vt = block_sum_d(vt);
-  vp = block_sum_d(vp);
-  if (threadIdx.x == 0) {
-    const double pAp = m2 * vp + vt;
+  const int halt = S->halt;
+  const double rr = S->rr;
+  const double vt = thread_sum_partials(pt, nt), vp = thread_sum_partials(pp, np);
+  const double pAp = block_sum_d(m2 * vp + vt);
+  if (threadIdx.x == 0 && !halt) {
     S->pAp = pAp;
     if (!(pAp > 0.0) || !isfinite(pAp)) {
       S->done = 2;
       S->halt = 1;
       return;
     }
-    const double a = S->rr / pAp;
+    const double a = rr / pAp;
     S->alpha = a;
-    S->alpha_dw = split_dev2(a);
-    S->malpha_dw = split_dev2(-a);
-    S->alpha_f = (float)a;
-    S->malpha_f = (float)-a;
+    const float2 d = split_dev2(a);  // d.x = (float)a
+    S->alpha_dw = d;
+    S->malpha_dw = make_float2(-d.x, -d.y);
+    S->alpha_f = d.x;
+    S->malpha_f = -d.x;
   }
 }
 
@@ -418,7 +399,7 @@ jqcd_status solve_staggered(GaugeEntry &G, double mass, const jqcd_solve_params 
         // hop applies the update and forms ||r||^2; beta; p = r + beta p, ||p||^2
         CKT(launch_stag_hop(G.g, 1, false, p, nullptr, t, U, 0.0, 1.0, part_t, s, &S->halt));
         note_launch();
-        CKT(launch_pdl(stag_alpha_kernel, 1, kReduceThreads, 0, s, part_t, nstag, part_p, nblas, m2, S));
+        CKT(launch_pdl(stag_alpha_kernel, 1, reduce_threads(std::max(nstag, nblas)), 0, s, part_t, nstag, part_p, nblas, m2, S));
         note_launch();
         CKT(launch_pdl(stag_hop_cg_kernel, nstag, kStagThreads, 0, s, G.g, t, p, xe, r, U, dw_split_host(m2),
                        dw_split_host(-1.0), S, part_t));

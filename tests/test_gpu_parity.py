@@ -238,6 +238,22 @@ def test_hop_eight_threads_per_site_edges(jq, dagger, prec, dims):
     g.free()
 
 
+@pytest.mark.parametrize("dims", [(16, 16, 32, 64), (16, 16, 32, 66), (32, 32, 32, 32), (32, 32, 32, 34)])
+def test_norm_partial_counts(jq, dims):
+    """The norm's single-block sum around its steps in block size: 2048, 2112,
+    4096 and 4352 partials of FP32 hops, against an FP64 sum over the output.
+    Bound: the FP32 sums of a site's 24 squares, all positive (24 x 6e-8)."""
+    jqcd, ctx = jq
+    import torch
+    g = ctx.gauge_upload(dims, synth.gauge(dims, "unit"))
+    inp = torch.randn(g.spinor_bytes(1) // 4, device="cuda").view(torch.uint8)
+    out, norm = g.empty(1), torch.zeros(1, dtype=torch.float64, device="cuda")
+    g.dslash_eo(1, 0, 0, inp, None, out, norm2=norm)
+    want = out.view(torch.float32).double().square().sum().item()
+    assert abs(norm.item() - want) <= 1.5e-6 * want
+    g.free()
+
+
 def test_current_stream_is_used(jq):
     """Without a stream argument a call goes to torch's current stream, also
     inside a stream context; streams, raw handles and buffers are all taken."""
