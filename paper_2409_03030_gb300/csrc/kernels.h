@@ -24,6 +24,11 @@ constexpr int kMixedBlock = 8;
 #ifndef JQCD_FIN_MAX_BLOCKS
 #define JQCD_FIN_MAX_BLOCKS 1024
 #endif
+// The same for the FP32 inner solver.
+#ifndef JQCD_FIN_MAX_BLOCKS_F32
+#define JQCD_FIN_MAX_BLOCKS_F32 128
+#endif
+static_assert(JQCD_FIN_MAX_BLOCKS_F32 <= JQCD_FIN_MAX_BLOCKS, "what the hops take");
 
 struct HopParams {
   void *out;

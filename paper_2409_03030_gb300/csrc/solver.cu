@@ -255,9 +255,15 @@ struct DwSystem {
 // JQCD_FIN_MAX_BLOCKS hop blocks) takes alpha and beta in the last block of
 // the hop that writes their partials (cg_steps.cuh) instead of a
 // single-block launch after it (measured on GB300: mixed FP16 solve at 16^4
-// 3.08 -> 2.83 ms).  The double-word iteration keeps the separate launches:
+// 3.00 -> 2.70 ms, at 8^4 1.95 -> 1.80 ms, equal from 512 blocks on).  With FP32
+// hops, whose blocks have twice the stores to fence before they count, only up
+// to 128 blocks: 8^4 1.96 -> 1.77 ms, 12^4 2.12 -> 2.10 ms, but with it 14^4
+// (151 blocks) takes 2.78 instead of 2.62 ms, 16^4 3.20 instead of 2.98 ms,
+// 16^3x32 4.28 instead of 4.03 ms.  The double-word iteration keeps the separate launches:
 // there the last-block form gained nothing at 16^4 and lost 2% at 8^4.
-static bool fuse_scalar_steps(int nb) { return nb <= JQCD_FIN_MAX_BLOCKS; }
+static bool fuse_scalar_steps(int hp, int nb) {
+  return nb <= (hp == PREC_F32 ? JQCD_FIN_MAX_BLOCKS_F32 : JQCD_FIN_MAX_BLOCKS);
+}
 
 // alpha = rr / <p, A p> from the partials of the hop just queued on s, on
 // the side stream: the next hop (t = H^dag_oe w) does not read alpha, so the
@@ -324,7 +330,7 @@ cudaError_t lp_eo_cg_iteration(GaugeEntry &G, int hp, int mk, double kappa, Solv
                                bool end, cudaStream_t s) {
   const double k2 = -kappa * kappa;
   const int nb = (int)hop_blocks(G.g.vh);
-  const bool fuse = fuse_scalar_steps(nb);
+  const bool fuse = fuse_scalar_steps(hp, nb);
   const int *guard = &S->halt;
   const int x_code = 16 * B.id + slot + 1;
   void *p = B.p[slot], *t = G.mt[mk], *w = G.mw[mk];

@@ -443,6 +443,21 @@ def test_cg_dw_eight_threads_per_site(jq, dims):
     g.free()
 
 
+@pytest.mark.parametrize("dims", [(16, 16, 16, 8), (8, 8, 8, 66)])
+def test_mixed_f32_scalar_step_forms(jq, dims):
+    """The FP32 inner CG with its scalar steps in the hops' last block (128 hop
+    blocks) and in launches of their own (132)."""
+    jqcd, ctx = jq
+    U = synth.gauge(dims, "expi", eps=0.3, seed=50)
+    b = synth.gaussian_spinor(dims, seed=51)
+    g = ctx.gauge_upload(dims, U)
+    x, info, st = g.cg_solve(b, 0.12, tol=1e-10, mode=jqcd.CG_MIXED_F32)
+    assert st == 0
+    res = system_residual(dims, U, b, x, 0.12, True)
+    assert res <= 1e-10 * (1 + 1e-6), res
+    g.free()
+
+
 @pytest.mark.parametrize("eo", [False, True])
 def test_cg_f64_config0_4x4(jq, eo):
     """Plain FP64 CG (JQCD_CG_F64: native FP64 hops, vectors and reductions):
