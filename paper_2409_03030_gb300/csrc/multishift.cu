@@ -305,20 +305,20 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
     return JQCD_EINVAL;
   }
   CKM(G.ensure_multishift(nshift));
-  // (after the caller's own allocations)
-  G.grow_ring(G.ms_r, spinor_parity_bytes(PREC_DW, G.g.vh), kMsBlock - 1);
   const int64_t vh = G.g.vh;
   const int64_t n = 12 * vh;  // complex double-word numbers of one parity
   const int nblas = (int)blas_blocks(n);
   const int nhop = (int)dw_hop_blocks(vh);  // partials of the double-word hops
   float4 *rhs = G.vec_even(G.vrhs), *pb = G.vec_even(G.vp), *Ap = G.vec_even(G.vAp);
-  // step j of a block writes its residual to ring[j]
-  const int nring = 1 + (int)G.ms_r.size();
-  float4 *ring[kMsBlock];
+  // step j of a block writes its residual to ring[j]: r, and the halves of the
+  // solver's vectors that the iterations leave alone (Ap is formed after them)
+  float4 *const ring[] = {G.vec_odd(G.vr), G.vec_odd(G.vp),   G.vec_even(G.vAp),  G.vec_odd(G.vAp),
+                          G.vec_odd(G.vw), G.vec_even(G.vt), G.vec_odd(G.vrhs), G.vec_even(G.vr)};
+  static_assert(sizeof ring / sizeof ring[0] == kMsBlock, "a place for each residual of a block");
+  static_assert(kMsCheckEvery % kMsBlock == 0, "x_i is final when the solve has halted");
   MsResiduals R;
-  memset(&R, 0, sizeof R);
-  for (int j = 0; j < nring; ++j) R.r[j] = ring[j] = j + 1 < nring ? (float4 *)G.ms_r[j] : G.vec_even(G.vr);
-  const float4 *r_last = ring[nring - 1];  // the newest residual
+  for (int j = 0; j < kMsBlock; ++j) R.r[j] = ring[j];
+  const float4 *r_last = ring[kMsBlock - 1];  // the newest residual
   MsSteps *B = G.ms_B;
   MsVectors V;
   memset(&V, 0, sizeof V);
@@ -336,7 +336,7 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
   CKM(launch_dw_norm2(rhs, n, G.partials, s));
   CKM(launch_ms_start(G.partials, nblas, S, P.tol * P.tol, P.maxiter, s));
   CKM(cudaMemsetAsync(&B->n, 0, sizeof B->n, s));
-  CKM(launch_dw_copy(ring[nring - 1], rhs, n, s));
+  CKM(launch_dw_copy(ring[kMsBlock - 1], rhs, n, s));
   CKM(launch_dw_copy(pb, rhs, n, s));
   for (int i = 0; i < nshift; ++i) {
     CKM(launch_dw_copy(V.p[i], rhs, n, s));
@@ -378,10 +378,9 @@ jqcd_status solve_multishift(GaugeEntry &G, const jqcd_solve_params &P, int nshi
   };
   for (;;) {
     for (int k = 0; k < kMsCheckEvery; ++k) {
-      const int slot = k % nring;
+      const int slot = k % kMsBlock;
       CKM(iteration(slot));
-      // (a poll ends a block too, so that x_i is final when the solve has halted)
-      if (slot + 1 == nring || k + 1 == kMsCheckEvery) CKM(launch_ms_steps(V, R, S, B, nblas, n, s));
+      if (slot + 1 == kMsBlock) CKM(launch_ms_steps(V, R, S, B, nblas, n, s));
     }
     CKM(cudaMemcpyAsync(H, S, sizeof(MsScalars), cudaMemcpyDeviceToHost, s));
     CKM(cudaStreamSynchronize(s));

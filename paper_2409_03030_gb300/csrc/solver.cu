@@ -26,12 +26,12 @@ namespace jqcd {
 
 namespace {
 constexpr int kCheckEvery = 8;
+static_assert(kCheckEvery % kMixedBlock == 0, "a poll finds x_s up to date");
 constexpr int kMaxRestarts = 8;
 }  // namespace
 
 GaugeEntry::~GaugeEntry() {
   for (void *p : device_allocs) cudaFree(p);
-  drop_rings();
   if (S_host) cudaFreeHost(S_host);
   if (ms_S_host) cudaFreeHost(ms_S_host);
   if (ev0) cudaEventDestroy(ev0);
@@ -44,36 +44,8 @@ GaugeEntry::~GaugeEntry() {
 cudaError_t GaugeEntry::alloc(void **p, size_t bytes) {
   *p = nullptr;
   cudaError_t e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
-  if (e == cudaErrorMemoryAllocation && drop_rings()) {
-    cudaGetLastError();
-    e = cudaMalloc(p, bytes < 256 ? 256 : bytes);
-  }
   if (e == cudaSuccess) device_allocs.push_back(*p);
   return e;
-}
-
-// Up to `most` vectors, each of no more than a sixteenth of the free memory.
-void GaugeEntry::grow_ring(std::vector<void *> &ring, size_t bytes, int most) {
-  while ((int)ring.size() < most) {
-    size_t free_b = 0, total = 0;
-    void *p = nullptr;
-    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess || bytes > free_b / 16 || cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return;
-    }
-    ring.push_back(p);
-  }
-}
-
-// (cudaFree waits for the device: nothing still reads them)
-bool GaugeEntry::drop_rings() {
-  bool any = false;
-  for (std::vector<void *> *r : {&ms_r, &mring[0], &mring[1]}) {
-    for (void *p : *r) cudaFree(p);
-    any = any || !r->empty();
-    r->clear();
-  }
-  return any;
 }
 
 cudaError_t GaugeEntry::ensure_canon() {
@@ -318,9 +290,20 @@ cudaError_t dw_eo_cg_iteration(GaugeEntry &G, double kappa, SolverScalars *S, cu
 // date (mixed_block_end_kernel) and writes p[0] of the next.
 struct InnerBlock {
   void *p[kMixedBlock];
-  int m;          // directions there is room for: steps of a block
   int id = 1;     // number of the block (27 bits)
 };
+
+// The directions beside mp lie in halves of the double-word vectors that a
+// mixed solve leaves alone: both of p (384 bytes per site of one parity), the
+// even one of t and the odd one of r (192 bytes each).  A direction takes 96
+// bytes per site (FP32) or 52 (FP16; 16-byte aligned, vh is a multiple of 8), so
+// four, two and one fit, and the solve needs no memory beyond its own vectors.
+InnerBlock inner_block(const GaugeEntry &G, int hp, int mk) {
+  static_assert(kMixedBlock == 8, "seven directions beside mp");
+  const size_t b = spinor_parity_bytes(hp, G.g.vh);
+  char *const p = (char *)G.vp, *const t = (char *)G.vec_even(G.vt), *const r = (char *)G.vec_odd(G.vr);
+  return InnerBlock{{G.mp[mk], p, p + b, p + 2 * b, p + 3 * b, t, t + b, r}};
+}
 
 // Step `slot` of a block of the inner CG of the mixed solver in hop precision
 // hp on the vectors p, t, w of that precision (FP32 xs and rs): the same order
@@ -364,7 +347,7 @@ cudaError_t lp_eo_cg_iteration(GaugeEntry &G, int hp, int mk, double kappa, Solv
   if (!fuse && (e = launch_mixed_beta(G.partials, nb, S, s))) return e;
   if (!end) return launch_mixed_xpay(hp, B.p[slot + 1], p, (const float4 *)G.mr, G.g.vh, S, s);
   MixedRing R;
-  for (int j = 0; j < kMixedBlock; ++j) R.p[j] = j < B.m ? B.p[j] : nullptr;
+  for (int j = 0; j < kMixedBlock; ++j) R.p[j] = B.p[j];
   e = launch_mixed_block_end(hp, (float4 *)G.mx, R, B.p[0], (const float4 *)G.mr, G.g.vh, B.id, S, s);
   B.id = B.id < (1 << 26) ? B.id + 1 : 1;
   return e;
@@ -441,9 +424,7 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
   InnerBlock IB;
   if (mixed) {
     CKS(G.ensure_mixed(hp));
-    G.grow_ring(G.mring[mk], spinor_parity_bytes(hp, vh), kMixedBlock - 1);
-    IB.m = 1 + (int)G.mring[mk].size();
-    for (int j = 0; j < IB.m; ++j) IB.p[j] = j ? G.mring[mk][j - 1] : G.mp[mk];
+    IB = inner_block(G, hp, mk);
   }
 
   CKS(cudaEventRecord(G.ev0, s));
@@ -505,8 +486,8 @@ static jqcd_status solve_cg(GaugeEntry &G, const jqcd_solve_params &P, cudaStrea
           CKS(launch_cg_beta(G.partials, nblas, S, s));
           CKS(launch_dw_xpay(G.vp, G.vr, A.n, S, s));
         } else {
-          const int slot = k % IB.m;
-          CKS(lp_eo_cg_iteration(G, hp, mk, P.kappa, S, IB, slot, slot + 1 == IB.m || k + 1 == kCheckEvery, s));
+          const int slot = k % kMixedBlock;
+          CKS(lp_eo_cg_iteration(G, hp, mk, P.kappa, S, IB, slot, slot + 1 == kMixedBlock, s));
         }
       }
       CKS(cudaMemcpyAsync(G.S_host, S, sizeof(SolverScalars), cudaMemcpyDeviceToHost, s));

@@ -26,11 +26,9 @@ struct GaugeEntry {
   float4 *vb = nullptr, *vsol = nullptr, *vr = nullptr, *vp = nullptr, *vAp = nullptr,
          *vw = nullptr, *vt = nullptr, *vrhs = nullptr;
   // mixed-precision inner vectors (even parity): x, r in FP32; p, w in the
-  // hop precision; t odd in the hop precision; mring: directions of a block of
-  // iterations beside mp
+  // hop precision; t odd in the hop precision
   void *mx = nullptr, *mr = nullptr, *mp[2] = {nullptr, nullptr}, *mw[2] = {nullptr, nullptr},
        *mt[2] = {nullptr, nullptr};
-  std::vector<void *> mring[2];
   // native FP64 solver vectors (whole lattice)
   double2 *fb = nullptr, *fsol = nullptr, *fr = nullptr, *fp = nullptr, *fAp = nullptr,
           *fw = nullptr, *ft = nullptr, *frhs = nullptr;
@@ -40,7 +38,6 @@ struct GaugeEntry {
   double *lcanon = nullptr;
   // multi-shift CG workspace: per-shift search directions and scalars
   std::vector<float4 *> ms_p, ms_x;  // ms_x: solutions of the host-buffer entry
-  std::vector<void *> ms_r;          // residuals of a block of iterations, beside vr
   MsScalars *ms_S = nullptr;
   MsSteps *ms_B = nullptr;
   MsScalars *ms_S_host = nullptr;  // pinned mirror
@@ -82,10 +79,6 @@ struct GaugeEntry {
   cudaError_t ensure_f64();
   cudaError_t ensure_force();
   cudaError_t ensure_multishift(int nshift);
-  // vectors that only make blocks of iterations longer: allocated while there
-  // is room for them, given back when another allocation runs out
-  void grow_ring(std::vector<void *> &ring, size_t bytes, int most);
-  bool drop_rings();
   cudaError_t ensure_staggered();
   cudaError_t ensure_hmc();
   // fermion-solve history of a trajectory: previous X, Y and two start vectors
