@@ -422,16 +422,7 @@ __global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS) hop_dwp8_k
 // less: 16^4 4.44 against 4.53 ms, 16^3x18 4.62 against 5.14 ms, 16^3x24 5.88
 // against 6.75 ms.  Four blocks per SM: with five (96 registers, 40 bytes
 // spilled) 8^4 takes 2.9 us, with three 12^4 5.6 us.
-bool dw_hop_split8(int64_t vh) {
-  static const int64_t max_vh = [] {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-      return (int64_t)0;
-    return (int64_t)sms * JQCD_DWP8_BLOCKS * kDwp8Sites;
-  }();
-  return vh <= max_vh;
-}
+static bool dw_hop_split8(int64_t vh, int64_t sms) { return vh <= sms * JQCD_DWP8_BLOCKS * kDwp8Sites; }
 
 // A one-thread grid of at most SMs x JQCD_DWP_SMALL_BLOCKS blocks is launched
 // with kDwpSmallSmem of shared memory, so that no SM takes a third block.
@@ -443,15 +434,8 @@ bool dw_hop_split8(int64_t vh) {
 // double-word solve 4.95 -> 4.71 ms.  All hops unrolled took 11.7 us when the
 // same kernel ran back to back, but its code (four kernels of about 90 KB)
 // misses the instruction cache in a real chain: 5.3 ms.
-bool dw_hop_small(int64_t vh) {
-  static const int64_t max_vh = [] {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-      return (int64_t)0;
-    return (int64_t)sms * JQCD_DWP_SMALL_BLOCKS * kDwp1Threads;
-  }();
-  return !dw_hop_split8(vh) && vh <= max_vh && vh <= JQCD_DWP_SMALL_MAX_VH;
+static bool dw_hop_small(int64_t vh, int64_t sms) {
+  return !dw_hop_split8(vh, sms) && vh <= sms * JQCD_DWP_SMALL_BLOCKS * kDwp1Threads && vh <= JQCD_DWP_SMALL_MAX_VH;
 }
 
 // Whole blocks per SM at one thread per site and the rest at eight, where the
@@ -463,25 +447,33 @@ bool dw_hop_small(int64_t vh) {
 // SM: 29.5 -> 32.0 us), and past JQCD_DWX_MAX_VH a rest no longer shows (24^3x48
 // 91.0 and 90.9 us; the solve at 24^3x32 21.9 and 22.1 ms).  Not below one
 // wave of one-thread blocks (16^3x24: 16.9 -> 17.1 us, 16^3x28 17.1 -> 19.3 us).
-unsigned dw_hop_whole(int64_t vh) {
-  static const int64_t sms = [] {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      return (int64_t)0;
-    return (int64_t)n;
-  }();
+static unsigned dw_hop_whole(int64_t vh, int64_t sms) {
   const int64_t wave = sms * JQCD_DWP_MIN_BLOCKS * kDwp1Threads;
   if (!sms || vh <= wave || vh > JQCD_DWX_MAX_VH) return 0;
   const int64_t blocks = (vh + kDwp1Threads - 1) / kDwp1Threads, whole = vh / kDwp1Threads / sms * sms;
   return 5 * (blocks - whole) <= 2 * sms ? (unsigned)whole : 0;
 }
 
-unsigned dw_hop_blocks(int64_t vh) {
-  const int64_t whole = dw_hop_whole(vh);
-  if (whole || dw_hop_split8(vh))
-    return (unsigned)(whole + (vh - whole * kDwp1Threads + kDwp8Sites - 1) / kDwp8Sites);
-  return (unsigned)((vh + kDwp1Threads - 1) / kDwp1Threads);
+// SMs of a device, 0 when they cannot be asked for (and asked for again then)
+static int device_sms(int device) {
+  static std::atomic<int> known[64];
+  const bool slot = device >= 0 && device < 64;
+  int n = slot ? known[device].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  if (device < 0 || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n < 1)
+    return 0;
+  if (slot) known[device].store(n, std::memory_order_relaxed);
+  return n;
+}
+
+DwHopForm dw_hop_form(int64_t vh) {
+  const int device = current_device();
+  const int64_t sms = device_sms(device);
+  const int64_t whole = dw_hop_whole(vh, sms);
+  const bool split8 = dw_hop_split8(vh, sms);
+  const int64_t blocks = whole || split8 ? whole + (vh - whole * kDwp1Threads + kDwp8Sites - 1) / kDwp8Sites
+                                         : (vh + kDwp1Threads - 1) / kDwp1Threads;
+  return DwHopForm{device, split8, dw_hop_small(vh, sms), (unsigned)whole, (unsigned)blocks};
 }
 
 unsigned hop_norm_partials(int prec, int64_t vh) {
@@ -492,23 +484,21 @@ unsigned hop_norm_partials(int prec, int64_t vh) {
 template <bool DAG, bool AXPY, bool NORM>
 static cudaError_t launch_hop_dw_t(const HopParams &P, cudaStream_t s) {
   note_launch();
-  static bool configured = false;  // one attribute call per instantiation
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(hop_dwp_kernel<DAG, AXPY, NORM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(hop_dwx_kernel<DAG, AXPY, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kDwp1Smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  const unsigned blocks = dw_hop_blocks(P.g.vh);
-  if (dw_hop_split8(P.g.vh))
-    return launch_pdl(hop_dwp8_kernel<DAG, AXPY, NORM>, blocks, kDwp8Threads, 0, s, P);
-  if (const unsigned whole = dw_hop_whole(P.g.vh))
-    return launch_pdl(hop_dwx_kernel<DAG, AXPY, NORM>, blocks, kDwp1Threads, kDwp1Smem, s, P, whole);
-  return launch_pdl(hop_dwp_kernel<DAG, AXPY, NORM>, blocks, kDwp1Threads,
-                    dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P);
+  static OncePerDevice configured;  // per instantiation
+  const DwHopForm F = dw_hop_form(P.g.vh);
+  const cudaError_t e = configured(F.device, [] {
+    const cudaError_t e1 = cudaFuncSetAttribute(
+        hop_dwp_kernel<DAG, AXPY, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
+    return e1 ? e1
+              : cudaFuncSetAttribute(hop_dwx_kernel<DAG, AXPY, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kDwp1Smem);
+  });
+  if (e) return e;
+  if (F.split8) return launch_pdl(hop_dwp8_kernel<DAG, AXPY, NORM>, F.blocks, kDwp8Threads, 0, s, P);
+  if (F.whole)
+    return launch_pdl(hop_dwx_kernel<DAG, AXPY, NORM>, F.blocks, kDwp1Threads, kDwp1Smem, s, P, F.whole);
+  return launch_pdl(hop_dwp_kernel<DAG, AXPY, NORM>, F.blocks, kDwp1Threads, F.small ? kDwpSmallSmem : kDwp1Smem, s,
+                    P);
 }
 
 static cudaError_t launch_hop_dw(const HopParams &P, bool dag, bool axpy, bool norm, cudaStream_t s) {

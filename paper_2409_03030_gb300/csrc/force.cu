@@ -332,13 +332,11 @@ cudaError_t launch_fermi_force(const Geom &g, const float4 *xe, const float4 *xo
                                const float4 *yo, const float4 *gauge_dw, double kappa, float4 *out,
                                cudaStream_t s) {
   if (g.vh >= kMaxHopSites) return cudaErrorInvalidValue;  // 32-bit offsets
-  static bool configured = false;  // 72 KB of dynamic shared memory needs the opt-in
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(force_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)kForceSmem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice configured;  // 72 KB of dynamic shared memory needs the opt-in
+  const cudaError_t e = configured(current_device(), [] {
+    return cudaFuncSetAttribute(force_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kForceSmem);
+  });
+  if (e != cudaSuccess) return e;
   note_launch();
   const float2 tk = dw_split_host(2.0 * kappa);
   const unsigned blocks = 2 * (unsigned)((g.vh + kForceThreads - 1) / kForceThreads);

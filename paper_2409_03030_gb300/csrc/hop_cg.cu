@@ -213,23 +213,23 @@ template <bool XUPD>
 static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x, const float4 *r_in, float4 *r,
                                   const float2 *alpha, cudaStream_t s) {
   note_launch();
-  static bool configured = false;  // one attribute call per instantiation
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kDwpSmallSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(hop_dwx_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kDwp1Smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  const unsigned blocks = dw_hop_blocks(P.g.vh);
-  if (dw_hop_split8(P.g.vh))
-    return launch_pdl(hop_dwp8_cg_kernel<XUPD>, blocks, kDwp8Threads, 0, s, P, p, x, r_in, r, alpha);
-  if (const unsigned whole = dw_hop_whole(P.g.vh))
-    return launch_pdl(hop_dwx_cg_kernel<XUPD>, blocks, kDwp1Threads, kDwp1Smem, s, P, whole, p, x, r_in, r, alpha);
-  return launch_pdl(hop_dwp_cg_kernel<XUPD>, blocks, kDwp1Threads,
-                    dw_hop_small(P.g.vh) ? kDwpSmallSmem : kDwp1Smem, s, P, p, x, r_in, r, alpha);
+  static OncePerDevice configured;  // per instantiation
+  const DwHopForm F = dw_hop_form(P.g.vh);
+  const cudaError_t e = configured(F.device, [] {
+    const cudaError_t e1 = cudaFuncSetAttribute(hop_dwp_cg_kernel<XUPD>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwpSmallSmem);
+    return e1 ? e1
+              : cudaFuncSetAttribute(hop_dwx_cg_kernel<XUPD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kDwp1Smem);
+  });
+  if (e) return e;
+  if (F.split8)
+    return launch_pdl(hop_dwp8_cg_kernel<XUPD>, F.blocks, kDwp8Threads, 0, s, P, p, x, r_in, r, alpha);
+  if (F.whole)
+    return launch_pdl(hop_dwx_cg_kernel<XUPD>, F.blocks, kDwp1Threads, kDwp1Smem, s, P, F.whole, p, x, r_in, r,
+                      alpha);
+  return launch_pdl(hop_dwp_cg_kernel<XUPD>, F.blocks, kDwp1Threads, F.small ? kDwpSmallSmem : kDwp1Smem, s, P, p, x,
+                    r_in, r, alpha);
 }
 
 cudaError_t launch_hop_dw_cg(const HopParams &P, const float4 *p, float4 *x, float4 *r,

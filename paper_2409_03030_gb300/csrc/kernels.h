@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "lattice.cuh"
 
 namespace jqcd {
@@ -10,6 +12,25 @@ namespace jqcd {
 // Process-wide count of kernel launches issued by the library (n may be
 // negative to take back launches recorded into a graph that is replayed).
 void note_launch(int64_t n = 1);
+
+// cudaSetDevice for this thread's work; current_device() is the device that the
+// thread chose last (asking the runtime instead, once per launch, made four
+// hops and a norm at 4^4 about 1 us slower).  Every entry that launches chooses.
+cudaError_t use_device(int device);
+int current_device();
+
+// What is set for a kernel on one device (its dynamic shared memory opt-in)
+// holds there alone: set() runs once for each device that launches it.
+struct OncePerDevice {
+  std::atomic<uint64_t> done{0};
+  template <typename F> cudaError_t operator()(int device, F &&set) {
+    const uint64_t bit = device >= 0 && device < 64 ? (uint64_t)1 << device : 0;  // others: each time
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = set();
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
 
 constexpr int kHopThreads = 128;
 inline unsigned hop_blocks(int64_t vh) { return (unsigned)((vh + kHopThreads - 1) / kHopThreads); }
@@ -51,24 +72,29 @@ struct HopParams {
 cudaError_t launch_hop(int prec, const HopParams &P, bool dag, bool axpy, bool norm,
                        cudaStream_t s);
 
-// The double-word hops run eight threads per output site on small lattices
-// (their grids, and per-block partial sums, are then one per 16 sites), where
-// one thread per site leaves the GPU short of warps.
-bool dw_hop_split8(int64_t vh);
-// Lattices one size up (at most JQCD_DWP_SMALL_MAX_VH sites per parity and a
-// one-thread grid that fits in one wave at a lower occupancy) limit the blocks
-// per SM.
+// Launch form of a double-word hop on vh sites per parity of the current
+// device (its rules follow the SM count: dslash.cu).
 #ifndef JQCD_DWP_SMALL_MAX_VH
 #define JQCD_DWP_SMALL_MAX_VH 65536
 #endif
-bool dw_hop_small(int64_t vh);
-// Whole blocks of 128 sites, one thread each, of a launch that gives its other
-// sites eight threads each (0: all sites are handled alike).
 #ifndef JQCD_DWX_MAX_VH
 #define JQCD_DWX_MAX_VH 163840
 #endif
-unsigned dw_hop_whole(int64_t vh);
-unsigned dw_hop_blocks(int64_t vh);                 // blocks of a double-word hop launch
+struct DwHopForm {
+  int device;       // the current device, -1 when it cannot be asked for
+  // small lattices: eight threads per output site (grids, and per-block partial
+  // sums, are then one per 16 sites), where one leaves the GPU short of warps
+  bool split8;
+  // one size up (a one-thread grid that fits in one wave at a lower
+  // occupancy): the blocks per SM are limited
+  bool small;
+  // whole blocks of 128 sites, one thread each, of a launch that gives its
+  // other sites eight threads each (0: all sites are handled alike)
+  unsigned whole;
+  unsigned blocks;  // of the launch
+};
+DwHopForm dw_hop_form(int64_t vh);
+inline unsigned dw_hop_blocks(int64_t vh) { return dw_hop_form(vh).blocks; }
 unsigned hop_norm_partials(int prec, int64_t vh);   // partials of a hop launch with norm
 
 // ---- layouts ----------------------------------------------------------------

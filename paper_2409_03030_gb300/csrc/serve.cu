@@ -132,7 +132,7 @@ struct Server {
 };
 
 void Server::loop(int li) {
-  cudaSetDevice(device);
+  use_device(device);
   ServeLane &L = lanes[li];
   BatchEngine *engine = L.engine.get();
   std::vector<int> finished;
