@@ -200,8 +200,9 @@ cudaError_t launch_lp_cg_t(const HopParams &P, float4 *rs, const SolverScalars *
 }  // namespace
 
 cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, float4 *rs, const SolverScalars *S, cudaStream_t s) {
-  note_launch();
+  if (P.g.vh >= kMaxHopSites) return cudaErrorInvalidValue;  // 32-bit neighbour offsets
   if (P.fin && (!P.fin_S || hop_blocks(P.g.vh) > (unsigned)JQCD_FIN_MAX_BLOCKS)) return cudaErrorInvalidValue;
+  note_launch();
   switch (prec) {
     case PREC_F32: return launch_lp_cg_t<PREC_F32>(P, rs, S, s);
     case PREC_F16N: return launch_lp_cg_t<PREC_F16N>(P, rs, S, s);
@@ -212,6 +213,7 @@ cudaError_t launch_hop_lp_cg(int prec, const HopParams &P, float4 *rs, const Sol
 template <bool XUPD>
 static cudaError_t launch_dw_cg_t(const HopParams &P, const float4 *p, float4 *x, const float4 *r_in, float4 *r,
                                   const float2 *alpha, cudaStream_t s) {
+  if (P.g.vh >= kMaxHopSites) return cudaErrorInvalidValue;  // 32-bit neighbour offsets
   note_launch();
   static OncePerDevice configured;  // per instantiation
   const DwHopForm F = dw_hop_form(P.g.vh);

@@ -69,7 +69,8 @@ __device__ __forceinline__ int64_t hop_neighbour(const Geom &g, int x, int y, in
 
 // A site of one parity and its neighbours in 32-bit arithmetic: a resident
 // gauge field takes 2688 bytes per site of one parity, so vh < 2^27 on any
-// device (launch_hop and the other entries refuse more) and 16 idx < 2^31.
+// device and 16 idx < 2^31.  The hops', fused hops' and force's launches refuse
+// more; a batch admits a solve by launch_hop on its field.
 constexpr int64_t kMaxHopSites = (int64_t)1 << 27;
 struct HopSite {
   unsigned idx, xh, y, z, t;

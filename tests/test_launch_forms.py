@@ -68,3 +68,16 @@ def test_launch_forms_follow_each_device(lib):
         ctx, gid = field(lib, device, (6, 6, 6, 270))
         assert lib.jqcd_dslash_eo(ctx, gid, DW, 0, 0, buf[0], None, buf[1], 0.0, 1.0, None, None) == 0
         assert lib.fake_last_grid() == (-(-vh // 16) if device == 0 else -(-vh // 128))
+
+
+@pytest.mark.parametrize("which", [0, 1, 2, 3])
+def test_fused_hops_refuse_fields_past_32_bit_offsets(lib, which):
+    """A site's byte offset in a 16-byte plane has 32 bits, bit 0 used: the
+    fused hops refuse 2^27 sites per parity, as the plain ones do, and launch
+    nothing."""
+    field(lib, 0, (4, 4, 4, 4))
+    before = lib.fake_launches()
+    assert lib.fake_launch_cg(which, ctypes.c_int64(2 ** 27)) == 1  # cudaErrorInvalidValue
+    assert lib.fake_launches() == before
+    assert lib.fake_launch_cg(which, ctypes.c_int64(2 ** 27 - 8)) == 0
+    assert lib.fake_launches() == before + 1
