@@ -267,7 +267,6 @@ __global__ void __launch_bounds__(kF64x8Threads, 4) hop_f64x8_kernel(const HopPa
   if (NORM) {
     const double s = block_sum_d(nrm);
     if (threadIdx.x == 0) P.partials[blockIdx.x] = s;
-    if (P.fin) hop_finish_scalars(P);  // uniform over the grid
   }
 }
 
@@ -517,10 +516,10 @@ static cudaError_t launch_hop_dw(const HopParams &P, bool dag, bool axpy, bool n
 
 cudaError_t launch_hop(int prec, const HopParams &P, bool dag, bool axpy, bool norm,
                        cudaStream_t s) {
-  // the last-block scalar step (FP64, FP32 and FP16 hops) needs the partials
-  // and at most JQCD_FIN_MAX_BLOCKS of them
-  if (P.fin && (prec == PREC_DW || !norm || !P.fin_S ||
-                hop_norm_partials(prec, P.g.vh) > (unsigned)JQCD_FIN_MAX_BLOCKS))
+  // the last-block scalar step (FP32 and FP16 hops) needs the partials and at
+  // most JQCD_FIN_MAX_BLOCKS of them
+  if (P.fin && ((prec != PREC_F32 && prec != PREC_F16N) || !norm || !P.fin_S ||
+                hop_blocks(P.g.vh) > (unsigned)JQCD_FIN_MAX_BLOCKS))
     return cudaErrorInvalidValue;
   if (P.g.vh >= kMaxHopSites) return cudaErrorInvalidValue;  // 32-bit neighbour offsets
   switch (prec) {
