@@ -81,3 +81,22 @@ def test_fused_hops_refuse_fields_past_32_bit_offsets(lib, which):
     assert lib.fake_launches() == before
     assert lib.fake_launch_cg(which, ctypes.c_int64(2 ** 27 - 8)) == 0
     assert lib.fake_launches() == before + 1
+
+
+@pytest.mark.parametrize("prec,dims,grid", [
+    (0, (6, 6, 6, 270), 1823),               # 29,160 sites: 16-site tiles
+    (0, (6, 6, 6, 274), 232),                # 29,592: one thread per site
+    (0, (6, 6, 6, 540), 456),                # 58,320: one wave of three blocks per SM
+    (0, (6, 6, 6, 542), 456 + 11),           # 58,536: the wave, and 168 sites in tiles
+    (0, (20, 18, 14, 26), 456 + 447),        # 65,520
+    (3, (10, 10, 10, 130), 4063),            # FP64, 65,000 sites: a tile per block
+    (3, (10, 10, 10, 134), 2094),            # 67,000: two
+    (3, (32, 32, 32, 34), 8704),             # 557,056: four
+])
+def test_edge_lattices_take_the_forms_they_stand_for(lib, prec, dims, grid):
+    """The lattices that the GPU tests take for the edges of the rules, on 152
+    SMs: the grid of the hop shows the form."""
+    ctx, gid = field(lib, 0, dims)
+    buf = [ctypes.c_void_p(1 << 20 << i) for i in range(3)]
+    assert lib.jqcd_dslash_eo(ctx, gid, prec, 0, 1, buf[0], buf[1], buf[2], 0.7, -0.12, None, None) == 0
+    assert lib.fake_last_grid() == grid
