@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(kLpThreads) batch_lp_hop_kernel(const BatchArg
 // Measured (ncu launch lists of the 24-solve batch, serialised): FP16 inner
 // operator 236 ms with one right-hand side per thread (5 blocks/SM), 267 ms
 // packed at 3 blocks/SM (155-168 registers), 222 ms packed at 4 blocks/SM
-// (128 registers, 8-160 B spilled); FP32 297, 300 and 277 ms.
+// (128 registers); FP32 297, 300 and 277 ms.  Spilled at 128 registers: 80 B
+// (FP16) and 60 B (FP32) in the last stage, at most 28 B in the others.
 #ifndef JQCD_BATCH_LP2_MIN_BLOCKS
 #define JQCD_BATCH_LP2_MIN_BLOCKS 4
 #endif

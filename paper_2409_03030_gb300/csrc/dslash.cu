@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(kHopThreads) hop_kernel(const HopParams P) {
 
 // Low-precision hop with the next hop's neighbour and link prefetched into
 // shared memory (hop_lp.cuh); same epilogue as hop_kernel.  HBM-bound (78.6 us
-// = 6.5 TB/s at 32^3x64); six blocks per SM (84 registers) measured best:
-// 27.9 us at 24^3x48 against 28.2 us with the compiler's 72-80 registers, 28.8
-// us cut for seven; mixed FP16 solve 14.11 -> 13.94 ms, at 32^3x64 40.0 ->
+// = 6.5 TB/s at 32^3x64); six blocks per SM (80 registers) measured best:
+// 27.9 us at 24^3x48 against 28.2 us with the compiler's own count (72, 80 with
+// the axpy, 96 with the norm too), 28.8 us cut for seven; mixed FP16 solve 14.11 -> 13.94 ms, at 32^3x64 40.0 ->
 // 39.6 ms.  Plain loads (hop_kernel) ran 25.6 us at 24^3x48 but 83.2 us at
 // 32^3x64 and 4.9 against 3.9 us at 16^4.
 template <int PREC, bool DAG, bool AXPY, bool NORM>
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kDwp1Threads, JQCD_DWP_MIN_BLOCKS)
 // Small lattices: eight threads per output site (dwp8_hop).  A hop there is a
 // latency chain, the loads' round trip and the arithmetic of as many hops as a
 // thread runs, on too few warps to hide it: with one hop per thread, 8^4 (two
-// threads: 5.3 us back to back) takes 2.7 us, 12^4 (8.3 us) 6.0 us.
+// threads: 5.3 us back to back) takes 2.7 us, 12^4 (8.3 us) 5.2 us.
 template <bool DAG, bool AXPY, bool NORM>
 __global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS) hop_dwp8_kernel(const HopParams P) {
   __shared__ ulonglong2 sm[6][kDwp8Threads];
@@ -445,7 +445,9 @@ static bool dw_hop_small(int64_t vh, int64_t sms) {
 // tiles last longer than the blocks they replace (20^3x24, 0.93 of a block per
 // SM: 29.5 -> 32.0 us), and past JQCD_DWX_MAX_VH a rest no longer shows (24^3x48
 // 91.0 and 90.9 us; the solve at 24^3x32 21.9 and 22.1 ms).  Not below one
-// wave of one-thread blocks (16^3x24: 16.9 -> 17.1 us, 16^3x28 17.1 -> 19.3 us).
+// wave of one-thread blocks, where only rests past the two fifths have been
+// measured (16^3x24, 0.53 of a block: 16.9 -> 17.1 us; 16^3x28, 0.95: 17.1 ->
+// 19.3 us).
 static unsigned dw_hop_whole(int64_t vh, int64_t sms) {
   const int64_t wave = sms * JQCD_DWP_MIN_BLOCKS * kDwp1Threads;
   if (!sms || vh <= wave || vh > JQCD_DWX_MAX_VH) return 0;

@@ -158,8 +158,9 @@ __global__ void __launch_bounds__(kDwp8Threads, JQCD_DWP8_MIN_BLOCKS)
 
 // Low-precision form for the inner CG: Ap = a w + b H^dag t in FP32 registers
 // (never rounded to the storage precision), then the FP32 update of the
-// inner residual rs with alpha_f and ||rs||^2 per hop block.  Cut for five blocks per SM (six
-// cost the FP16 solve 1.5% at 24^3x48).
+// inner residual rs with alpha_f and ||rs||^2 per hop block.  Five blocks per SM:
+// 96 registers, which the compiler also takes without the bound; cut for six
+// the FP16 solve took 1.5% longer at 24^3x48.
 template <int PREC>
 __global__ void __launch_bounds__(kHopThreads, 5)
     hop_lp_cg_kernel(const HopParams P, float4 *__restrict__ rs, const SolverScalars *__restrict__ S) {

@@ -335,6 +335,7 @@ __device__ __forceinline__ void dwp_hop_site(float4 *dsm, const float4 *in, cons
 // 5.2).  A hop's latency chain is then one hop long.
 constexpr int kDwp8Sites = 16;
 constexpr int kDwp8Threads = 8 * kDwp8Sites;
+static_assert(kDwp1Threads == kDwp8Threads, "the blocks of hop_dwx_kernel run either form");
 
 // This thread's r = W h into sm[3 s + c][thread] (see above); idx: its site.
 template <bool DAG>

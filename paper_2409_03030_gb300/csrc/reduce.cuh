@@ -1,5 +1,5 @@
-// Deterministic block reductions: a fixed warp-shuffle tree, then warps summed
-// in order by thread 0.  Per-block results go to a partials array that a
+// Deterministic block reductions: a fixed warp-shuffle tree, then the same over
+// the warps' values in the first warp.  Per-block results go to a partials array that a
 // single-block kernel later sums in a fixed order, so a reduction over a
 // given launch shape always rounds the same way.
 #pragma once

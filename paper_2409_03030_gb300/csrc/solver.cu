@@ -219,10 +219,6 @@ struct DwSystem {
   }
 };
 
-// One double-word CG iteration on the even-odd system, p -> (x, r, p):
-// w = Mhat p with ||w||^2 = <p, Mhat^dag Mhat p> fused into the second hop,
-// alpha, then the last hop of Mhat^dag w applies x += alpha p, r -= alpha Ap
-// and forms ||r||^2 itself (Ap is never stored), beta, p = r + beta p.
 // The inner solver of the mixed CG on small grids (at most
 // JQCD_FIN_MAX_BLOCKS hop blocks) takes alpha and beta in the last block of
 // the hop that writes their partials (cg_steps.cuh) instead of a
@@ -231,8 +227,8 @@ struct DwSystem {
 // hops, whose blocks have twice the stores to fence before they count, only up
 // to 128 blocks: 8^4 1.96 -> 1.77 ms, 12^4 2.12 -> 2.10 ms, but with it 14^4
 // (151 blocks) takes 2.78 instead of 2.62 ms, 16^4 3.20 instead of 2.98 ms,
-// 16^3x32 4.28 instead of 4.03 ms.  The double-word iteration keeps the separate launches:
-// there the last-block form gained nothing at 16^4 and lost 2% at 8^4.
+// 16^3x32 4.28 instead of 4.03 ms.  The double-word iteration keeps the separate
+// launches: there the last-block form gained nothing at 16^4 and lost 2% at 8^4.
 static bool fuse_scalar_steps(int hp, int nb) {
   return nb <= (hp == PREC_F32 ? JQCD_FIN_MAX_BLOCKS_F32 : JQCD_FIN_MAX_BLOCKS);
 }
@@ -255,6 +251,10 @@ static cudaError_t alpha_join(GaugeEntry &G, cudaStream_t s) {
   return cudaStreamWaitEvent(s, G.ev_join, 0);
 }
 
+// One double-word CG iteration on the even-odd system, p -> (x, r, p):
+// w = Mhat p with ||w||^2 = <p, Mhat^dag Mhat p> fused into the second hop,
+// alpha, then the last hop of Mhat^dag w applies x += alpha p, r -= alpha Ap
+// and forms ||r||^2 itself (Ap is never stored), beta, p = r + beta p.
 cudaError_t dw_eo_cg_iteration(GaugeEntry &G, double kappa, SolverScalars *S, cudaStream_t s) {
   const double k2 = -kappa * kappa;
   const int nb = (int)dw_hop_blocks(G.g.vh);
