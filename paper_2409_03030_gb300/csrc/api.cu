@@ -33,18 +33,6 @@ std::atomic<uint64_t> g_launches{0};
 }
 void jqcd::note_launch(int64_t n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
-static thread_local int t_device = -1;
-cudaError_t jqcd::use_device(int device) {
-  const cudaError_t e = cudaSetDevice(device);
-  t_device = e == cudaSuccess ? device : -1;
-  return e;
-}
-int jqcd::current_device() {
-  int device = t_device;
-  if (device < 0 && cudaGetDevice(&device) != cudaSuccess) device = -1;
-  return device;
-}
-
 struct jqcd_ctx {
   int device = 0;
   int sm_count = 0;
@@ -91,7 +79,7 @@ jqcd_status cuda_fail(jqcd_ctx *ctx, cudaError_t e, const char *where) {
 jqcd_status check_ctx(jqcd_ctx *ctx) {
   if (!ctx) return JQCD_EINVAL;
   if (ctx->poisoned) return fail(ctx, JQCD_ECUDA, "context poisoned by an earlier CUDA error");
-  cudaError_t e = use_device(ctx->device);
+  cudaError_t e = cudaSetDevice(ctx->device);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaSetDevice");
   return JQCD_OK;
 }
@@ -149,7 +137,7 @@ jqcd_status jqcd_init(int device, jqcd_ctx **out) {
     return JQCD_ECUDA;
   }
   if (device < 0 || device >= n) return JQCD_EINVAL;
-  if (use_device(device) != cudaSuccess) return JQCD_ECUDA;
+  if (cudaSetDevice(device) != cudaSuccess) return JQCD_ECUDA;
   std::unique_ptr<jqcd_ctx> ctx(new (std::nothrow) jqcd_ctx());
   if (!ctx) return JQCD_ENOMEM;
   ctx->device = device;
@@ -162,7 +150,7 @@ jqcd_status jqcd_init(int device, jqcd_ctx **out) {
 jqcd_status jqcd_finalize(jqcd_ctx *ctx) {
   JQCD_RANGE();
   if (!ctx) return JQCD_EINVAL;
-  use_device(ctx->device);
+  cudaSetDevice(ctx->device);
   if (ctx->server) {
     std::string err;
     serve_destroy(ctx->server, nullptr, &err);
@@ -221,7 +209,7 @@ jqcd_status jqcd_gauge_free(jqcd_ctx *ctx, uint64_t gauge_id) {
     return fail(ctx, JQCD_EBUSY, "gauge %llu has requests in flight", (unsigned long long)gauge_id);
   if (it == ctx->gauges.end()) return fail(ctx, JQCD_ENOTFOUND, "unknown gauge id %llu",
                                            (unsigned long long)gauge_id);
-  use_device(ctx->device);
+  cudaSetDevice(ctx->device);
   if (!ctx->poisoned) cudaDeviceSynchronize();
   ctx->gauges.erase(it);
   return JQCD_OK;

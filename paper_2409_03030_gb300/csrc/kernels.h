@@ -13,11 +13,17 @@ namespace jqcd {
 // negative to take back launches recorded into a graph that is replayed).
 void note_launch(int64_t n = 1);
 
-// cudaSetDevice for this thread's work; current_device() is the device that the
-// thread chose last (asking the runtime instead, once per launch, made four
-// hops and a norm at 4^4 about 1 us slower).  Every entry that launches chooses.
-cudaError_t use_device(int device);
-int current_device();
+// The current device, -1 when it cannot be asked for.  Asked for at each launch
+// (17 ns) where there is more than one.
+inline int current_device() {
+  static const bool single = [] {
+    int n = 0;
+    return cudaGetDeviceCount(&n) == cudaSuccess && n == 1;
+  }();
+  if (single) return 0;
+  int device = -1;
+  return cudaGetDevice(&device) == cudaSuccess ? device : -1;
+}
 
 // What is set for a kernel on one device (its dynamic shared memory opt-in)
 // holds there alone: set() runs once for each device that launches it.

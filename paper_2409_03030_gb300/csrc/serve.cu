@@ -132,7 +132,7 @@ struct Server {
 };
 
 void Server::loop(int li) {
-  use_device(device);
+  cudaSetDevice(device);
   ServeLane &L = lanes[li];
   BatchEngine *engine = L.engine.get();
   std::vector<int> finished;
